@@ -15,20 +15,70 @@ int field_blocks() { return 152 * 4; }  // 4 blocks per SM of the 152-SM GB300
 // ------------------------------------------------------------------------------------
 // Finishing reduction of per-block partial sums
 // ------------------------------------------------------------------------------------
-constexpr int kFinishThreads = 256;  // one block (1024 threads measured slower: 17 vs 14 us)
+// The rows are summed by one cluster of up to eight blocks: each takes a contiguous share of
+// the rows, eight threads a row (one 64-byte row per eight lanes, so a warp reads 256
+// contiguous bytes), and hands its five sums to block 0 through distributed shared memory,
+// which adds them in block order.  The order depends on the row count alone.  One block
+// reading every row by itself was bound by its own loads: 34 us at 8192 rows, 6 us here (the
+// scalar tail is about 5 us of that); with few rows one block is enough and the cluster is 1.
+constexpr int kFinishThreads = 256;
+constexpr int kFinishClusterMax = 8;
+constexpr int kFinishRowsPerBlock = 256;  // rows that make another block worth its hand-over
+static int finish_cluster(int nblocks) {
+  int c = 1;
+  while (c < kFinishClusterMax && c * kFinishRowsPerBlock < nblocks) c *= 2;
+  return c;
+}
+
+// Sums of the rows into tot of cluster block 0 (all its threads may read it on return).
+// Returns whether this block is block 0.
+__device__ __forceinline__ bool finish_rows(const double* __restrict__ partials, int nblocks, double (&tot)[kNumSums]) {
+  __shared__ double warp_s[kFinishThreads / 32][8];
+  __shared__ double part_s[kFinishClusterMax][8];
+  const int rank = blockIdx.x, nb = gridDim.x;
+  const int tid = threadIdx.x, comp = tid & 7, lane = tid & 31, warp = tid >> 5;
+  const int r0 = (int)((long long)rank * nblocks / nb), r1 = (int)((long long)(rank + 1) * nblocks / nb);
+  double s = 0.0;
+  if (comp < kNumSums) {
+#pragma unroll 8
+    for (int r = r0 + (tid >> 3); r < r1; r += kFinishThreads / 8) s += partials[(long long)r * kPartialStride + comp];
+  }
+  s += __shfl_down_sync(0xffffffffu, s, 16);
+  s += __shfl_down_sync(0xffffffffu, s, 8);
+  if (lane < 8) warp_s[warp][lane] = s;
+  __syncthreads();
+  if (nb > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  if (tid < kNumSums) {
+    double t = warp_s[0][tid];
+#pragma unroll
+    for (int w = 1; w < kFinishThreads / 32; ++w) t += warp_s[w][tid];
+    if (nb == 1) {
+      part_s[0][tid] = t;
+    } else {
+      unsigned dst;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+                   : "=r"(dst)
+                   : "r"((unsigned)__cvta_generic_to_shared(&part_s[rank][tid])), "r"(0));
+      asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(dst), "d"(t) : "memory");
+    }
+  }
+  if (nb > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  else __syncthreads();
+  if (rank != 0) return false;
+#pragma unroll
+  for (int i = 0; i < kNumSums; ++i) {
+    double t = part_s[0][i];
+    for (int b = 1; b < nb; ++b) t += part_s[b][i];
+    tot[i] = t;
+  }
+  return true;
+}
 
 __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const double* __restrict__ partials, int nblocks,
                                                      DevScalars* sc, int set_scale, int interval,
                                                      double dtau) {
-  __shared__ double red_s[32 * kNumSums];
-  __shared__ double tot[kNumSums];
-  double s[kNumSums] = {0, 0, 0, 0, 0};
-#pragma unroll 4
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-    for (int i = 0; i < kNumSums; ++i) s[i] += partials[(long long)b * kPartialStride + i];
-  block_sum_store<kNumSums>(s, red_s, tot);
-  __syncthreads();
+  double tot[kNumSums];
+  if (!finish_rows(partials, nblocks, tot)) return;
   if (threadIdx.x == 0) {
     const double nrm = tot[0];
     for (int i = 0; i < kNumSums; ++i) sc->sums[i] = tot[i];
@@ -67,10 +117,26 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const double* __
   }
 }
 
+// One cluster of c blocks.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_cluster(void (*kern)(KArgs...), int c, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(c);
+  cfg.blockDim = dim3(kFinishThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = c;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 cudaError_t launch_finish(const double* partials, int nblocks, DevScalars* sc, int set_scale, cudaStream_t st,
                           int interval, double dtau) {
-  finish_kernel<<<1, kFinishThreads, 0, st>>>(partials, nblocks, sc, set_scale, interval, dtau);
-  return cudaGetLastError();
+  return launch_cluster(finish_kernel, finish_cluster(nblocks), st, partials, nblocks, sc, set_scale, interval, dtau);
 }
 
 // ------------------------------------------------------------------------------------
@@ -134,15 +200,8 @@ cudaError_t launch_dots(const cpx<R>* const* basis, int nb, const cpx<R>* w, lon
 // coef_out: [Re c0, Im c0, Re c1, Im c1, |w|^2, 1/|w|]
 __global__ void __launch_bounds__(kFinishThreads) finish_dots_kernel(const double* __restrict__ partials, int nblocks,
                                                           double* coef_out) {
-  __shared__ double red_s[32 * kNumSums];
-  __shared__ double tot[kNumSums];
-  double s[kNumSums] = {0, 0, 0, 0, 0};
-#pragma unroll 4
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-    for (int i = 0; i < kNumSums; ++i) s[i] += partials[(long long)b * kPartialStride + i];
-  block_sum_store<kNumSums>(s, red_s, tot);
-  __syncthreads();
+  double tot[kNumSums];
+  if (!finish_rows(partials, nblocks, tot)) return;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kNumSums; ++i) coef_out[i] = tot[i];
     coef_out[5] = tot[4] > 0 ? 1.0 / sqrt(tot[4]) : 0.0;
@@ -151,8 +210,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_dots_kernel(const doubl
 
 cudaError_t launch_finish_dots(const double* partials, int nblocks, int nb, double* coef_out, cudaStream_t st) {
   (void)nb;
-  finish_dots_kernel<<<1, kFinishThreads, 0, st>>>(partials, nblocks, coef_out);
-  return cudaGetLastError();
+  return launch_cluster(finish_dots_kernel, finish_cluster(nblocks), st, partials, nblocks, coef_out);
 }
 
 // w = src - sum_j c_j v_j with c_j from device memory, then the sums <v_j|w> and <w|w> of
