@@ -42,7 +42,7 @@ TRAFFIC_FILES = {
     "fft": (os.path.join(ROOT, "profiles", "ncu_traffic_fft_step_n256.json"),
             ("qf_fft_impl.cuh", "qf_common.cuh", "qf_fft2.cuh")),
     "stencil": (os.path.join(ROOT, "profiles", "ncu_traffic_fdtd_step_n256.json"),
-                ("qf_stencil.cu", "qf_stencil_tma.cuh", "qf_stencil_tb.cuh", "qf_common.cuh")),
+                ("qf_stencil.cu", "qf_stencil_flat.cuh", "qf_stencil_tb.cuh", "qf_common.cuh")),
 }
 FALLBACK_HBM_GBS = 6800.0
 

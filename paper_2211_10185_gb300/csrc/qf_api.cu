@@ -2,7 +2,7 @@
 // device workspace, the step loop with its checks and snapshots, Gram-Schmidt excited
 // states and parity projection.  Every arithmetic step on fields runs in the kernels of
 // qf_fft_impl.cuh (four-pass FFT step), qf_fft2.cuh (two-pass step, N = 128 and 256),
-// qf_stencil_tma.cuh / qf_stencil_tb.cuh (FDTD steps) and qf_fields.cu; this file only
+// qf_stencil_flat.cuh / qf_stencil_tb.cuh (FDTD steps) and qf_fields.cu; this file only
 // sequences them.
 #include <math.h>
 
@@ -21,17 +21,14 @@
 #include "qf_stencil_tb.cuh"
 
 namespace qf {
-bool encode_stencil_map(CUtensorMap* map, void* field, int n, bool c64);
-bool encode_tb_map(CUtensorMap* map, void* field, int n);
 bool fft2_supported(int n);
 int fft2_final_blocks(int n);
 int fft2_measure_blocks(int n);
 cudaError_t launch_fft2_group_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
-cudaError_t launch_stencil_tb(const StencilTbArgs& g, cudaStream_t st);
-cudaError_t launch_stencil_tb_group(const StencilTbGroup& g, cudaStream_t st);
+cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st);
 cudaError_t launch_bounded_wait_probe(int* err, cudaStream_t st);
 template <typename R>
-cudaError_t launch_stencil_tma(const StencilTmaGroup<R>& g, cudaStream_t st);
+cudaError_t launch_stencil(const StencilGroup<R>& g, cudaStream_t st);
 template <typename R>
 cudaError_t launch_pack_f64(cpx<R>* dst, const double* re, const double* im, long long n, cudaStream_t st);
 }  // namespace qf
@@ -95,7 +92,7 @@ static Layout make_layout(const qf_lattice_desc& d) {
     if (fb > mb) mb = fb;
   }
   if (d.prec == QF_PREC_C64 && fft2_supported(d.n) && fft2_measure_blocks(d.n) > mb) mb = fft2_measure_blocks(d.n);
-  int sb = d.prec == QF_PREC_C64 ? stencil_blocks<float>(d.n) : stencil_blocks<double>(d.n);
+  const int sb = stencil_blocks(d.n);
   if (sb > mb) mb = sb;
   L.max_blocks = mb;
   L.partials = off;
@@ -149,19 +146,13 @@ struct qf_lattice {
   bool xfwd_valid = false;
   // CUDA graphs of the check_every-1 steps that follow a check (see run_chunk_graph)
   struct Graph {
-    int check_every, live, tblock, kzero;
+    int check_every, live, tblock;
     cudaGraphExec_t exec;
     int flips;         // FDTD buffer swaps done by the replay
     int64_t launches;  // kernels in the graph
   };
   std::vector<Graph> graphs;
   bool use_graphs = true;
-  // tensor maps of the two field buffers for the TMA-staged stencil (one-site halo) and
-  // for the two-step stencil (two-site halo, complex FP32)
-  CUtensorMap fmap[2];
-  bool fmap_ok = false;
-  CUtensorMap tbmap[2];
-  bool tbmap_ok = false;
   // FDTD steps fused per pass (1 or 2) and whether the live field is known to be zero on
   // the Dirichlet planes (it is after any FDTD step), which the two-step kernel needs
   int tblock = 2;
@@ -317,10 +308,6 @@ extern "C" qf_status qf_create_lattice(const qf_lattice_desc* desc, void* dev_ws
     delete lat;
     return QF_ECUDA;
   }
-  lat->fmap_ok = encode_stencil_map(&lat->fmap[0], lat->field(0), desc->n, desc->prec == QF_PREC_C64) &&
-                 encode_stencil_map(&lat->fmap[1], lat->field(1), desc->n, desc->prec == QF_PREC_C64);
-  lat->tbmap_ok = desc->prec == QF_PREC_C64 && encode_tb_map(&lat->tbmap[0], lat->field(0), desc->n) &&
-                  encode_tb_map(&lat->tbmap[1], lat->field(1), desc->n);
   *out = lat;
   return QF_OK;
 }
@@ -554,68 +541,20 @@ static StencilArgs<R> stencil_args(qf_lattice* lat, void* in, void* out, bool wr
                         write ? 1 : 0, reduce ? 1 : 0};
 }
 
-// Appends lattice `lat` (input field `in`) to a TMA stencil group; the tensor map of a
-// field buffer is cached, others (state slots) are encoded on the spot.
+// Appends lattice `lat` (input field `in`) to a stencil group.
 template <typename R>
 static bool stencil_group_member(qf_lattice* lat, void* in, void* out, bool write, bool reduce, const double* scale,
-                                 StencilTmaGroup<R>& g, bool first = true, int zc = kStencilZChunks[2]) {
-  if (first) {
-    g.count = 0;
-    g.err = &lat->sc()->err[0];
-  }
+                                 StencilGroup<R>& g, bool first = true) {
+  if (first) g.count = 0;
   const int i = g.count;
   if (i >= kGroupMax) return false;
   g.nm[i] = lat->d.n;
-  g.zcm[i] = zc;
-  if (in == lat->field(0) && lat->fmap_ok) g.map[i] = lat->fmap[0];
-  else if (in == lat->field(1) && lat->fmap_ok) g.map[i] = lat->fmap[1];
-  else if (!encode_stencil_map(&g.map[i], in, lat->d.n, lat->c64())) return false;
   g.a[i] = stencil_args<R>(lat, in, out, write, reduce, scale);
   g.count = i + 1;
   return true;
 }
 
-// ---- autotuner: z-chunk of the TMA stencil, per (N, precision), process-wide ----------
-static std::mutex g_tune_mu;
-static std::vector<std::pair<long long, int>> g_tuned_zc;  // key (n * 2 + c64) -> zc
-
-template <typename R>
-static int tuned_zchunk(qf_lattice* lat) {
-  const long long key = (long long)lat->d.n * 2 + (lat->c64() ? 1 : 0);
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    for (auto& kv : g_tuned_zc)
-      if (kv.first == key) return kv.second;
-  }
-  // time one step (psi -> scratch, no sums) for each candidate; the scratch field is
-  // overwritten by the real step afterwards
-  int best = kStencilZChunks[2];
-  float best_ms = 1e30f;
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return best;
-  for (int zc : kStencilZChunks) {
-    StencilTmaGroup<R> g;
-    if (!stencil_group_member<R>(lat, lat->psi(), lat->tmp(), true, false, &lat->sc()->scale[0], g, true, zc)) break;
-    float ms = 0, tot = 0;
-    bool ok = launch_stencil_tma<R>(g, lat->st) == cudaSuccess;  // warm-up
-    for (int rep = 0; rep < 3 && ok; ++rep) {
-      ok = cudaEventRecord(e0, lat->st) == cudaSuccess && launch_stencil_tma<R>(g, lat->st) == cudaSuccess &&
-           cudaEventRecord(e1, lat->st) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
-           cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
-      tot += ms;
-    }
-    lat->launches += 4;
-    if (ok && tot < best_ms) {
-      best_ms = tot;
-      best = zc;
-    }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tuned_zc.push_back({key, best});
-  return best;
-}
+static std::mutex g_tune_mu;  // the autotuners' tables
 
 // ---- autotuner: tile geometry and radix plan of the complex-FP32 four-pass FFT, per N ---
 // On the first four-pass FFT step of a size, every variant (two tile geometries, times two
@@ -669,22 +608,10 @@ static void tune_fft_tiles(qf_lattice* lat) {
   lat->xfwd_valid = false;  // the scratch field was overwritten
 }
 
-// Reads and clears the bounded-wait failure flag of a lattice.
-static qf_status check_device_error(qf_lattice* lat) {
-  int err = 0;
-  QF_CUDA(lat, cudaMemcpyAsync(&err, &lat->sc()->err[0], sizeof(int), cudaMemcpyDeviceToHost, lat->st));
-  QF_CUDA(lat, cudaStreamSynchronize(lat->st));
-  if (err) {
-    QF_CUDA(lat, cudaMemsetAsync(&lat->sc()->err[0], 0, sizeof(int), lat->st));
-    return fail(lat, QF_ETIMEOUT, "a bounded device wait ran out (copy engine did not complete)");
-  }
-  return QF_OK;
-}
-
 // ---- two FDTD steps per pass (complex FP32) ----------------------------------------------
-static void tb_args(qf_lattice* lat, const double* scale, int nzb, StencilTbArgs& g) {
+static void tb_args(qf_lattice* lat, const double* scale, StencilTbArgs& g) {
   const double a = lat->d.a, m = lat->mass, dt = lat->dtau;
-  g.map = lat->tbmap[lat->live];
+  g.in = reinterpret_cast<const cpx<float>*>(lat->psi());
   g.out = reinterpret_cast<cpx<float>*>(lat->tmp());
   g.v = lat->ws + lat->L.v;
   g.v_real = lat->v_real ? 1 : 0;
@@ -692,78 +619,25 @@ static void tb_args(qf_lattice* lat, const double* scale, int nzb, StencilTbArgs
   g.half_dtau = (float)(0.5 * dt);
   g.kd = (float)(dt / (2.0 * m * a * a));
   g.scale = scale;
+  g.scale2 = &lat->sc()->scale[2];
   g.n = lat->d.n;
-  g.nzb = nzb;
-  g.err = &lat->sc()->err[0];
-}
-
-static std::vector<std::pair<long long, int>> g_tuned_tb;  // key n -> z-chunks per tile
-
-// Number of z-chunks per column tile of the two-step kernel, per N, timed on first use
-// (psi -> scratch; the scratch field is overwritten by the real pass afterwards) among
-// chunks of about 64, 32 and 16 planes and the counts that make the grid about 1-4 full
-// waves of two resident blocks per SM.  Must not run during a capture.
-static int tuned_tb_zchunk(qf_lattice* lat) {
-  const int n = lat->d.n;
-  const long long key = n;
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    for (auto& kv : g_tuned_tb)
-      if (kv.first == key) return kv.second;
-  }
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int tiles = ((n + TB_X - 1) / TB_X) * ((n + TB_Y - 1) / TB_Y);
-  std::vector<int> cand = {(n + 63) / 64, (n + 31) / 32, (n + 15) / 16};
-  for (int w = 1; w <= 4; ++w) {
-    cand.push_back(w * 2 * sms / tiles);
-    cand.push_back((w * 2 * sms + tiles - 1) / tiles);
-  }
-  std::sort(cand.begin(), cand.end());
-  cand.erase(std::unique(cand.begin(), cand.end()), cand.end());
-  int best = (n + 31) / 32;
-  float best_ms = 1e30f;
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return best;
-  for (int nzb : cand) {
-    if (nzb < 1 || nzb > n) continue;
-    StencilTbArgs g;
-    tb_args(lat, &lat->sc()->scale[0], nzb, g);
-    float ms = 0, tot = 0;
-    bool ok = launch_stencil_tb(g, lat->st) == cudaSuccess;  // warm-up
-    for (int rep = 0; rep < 3 && ok; ++rep) {
-      ok = cudaEventRecord(e0, lat->st) == cudaSuccess && launch_stencil_tb(g, lat->st) == cudaSuccess &&
-           cudaEventRecord(e1, lat->st) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
-           cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
-      tot += ms;
-    }
-    lat->launches += 4;
-    if (ok && tot < best_ms) {
-      best_ms = tot;
-      best = nzb;
-    }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tuned_tb.push_back({key, best});
-  return best;
+  g.nzb = stencil_tb_chunks(g.n);
 }
 
 // Whether steps t and t+1 may run as one two-step pass: complex FP32 FDTD with blocking
 // on and a clean live field, no check at t or t+1 and no snapshot after step t.
 static bool fuse_pair(const qf_lattice* lat, int64_t t, int check_every, int snap_every) {
-  if (lat->kinetic != QF_KIN_FDTD || !lat->c64() || lat->tblock < 2 || !lat->clean || !lat->tbmap_ok) return false;
-  if (lat->kcur != 0) return false;  // the second step of a pair applies no scale
+  if (lat->kinetic != QF_KIN_FDTD || !lat->c64() || lat->tblock < 2 || !lat->clean) return false;
   if (check_every > 0 && (t % check_every == 0 || (t + 1) % check_every == 0)) return false;
   if (snap_every > 0 && (t + 1) % snap_every == 0) return false;
   return true;
 }
 
 // psi_{t+2} into the scratch field; `scale` renormalises the first of the two steps.
-static cudaError_t fdtd_pair(qf_lattice* lat, const double* scale, int nzb) {
-  StencilTbArgs g;
-  tb_args(lat, scale, nzb, g);
+static cudaError_t fdtd_pair(qf_lattice* lat, const double* scale) {
+  StencilTbGroup g;
+  g.count = 1;
+  tb_args(lat, scale, g.m[0]);
   return launch(lat, K_STENCIL_2STEP, [&] { return launch_stencil_tb(g, lat->st); });
 }
 
@@ -773,16 +647,16 @@ static cudaError_t kinetic_pass(qf_lattice* lat, void* in, void* out, bool write
                                 int* nblocks) {
   const int n = lat->d.n;
   if (lat->kinetic == QF_KIN_FDTD) {
-    const int zc = lat->c64() ? tuned_zchunk<float>(lat) : tuned_zchunk<double>(lat);
-    if (nblocks) *nblocks = stencil_blocks<float>(n, zc);
+    if (nblocks) *nblocks = stencil_blocks(n);
+    const int kind = write ? K_STENCIL : K_STENCIL_SUMS;
     if (lat->c64()) {
-      StencilTmaGroup<float> g;
-      if (!stencil_group_member(lat, in, out, write, reduce, scale, g, true, zc)) return cudaErrorInvalidValue;
-      return launch(lat, write ? K_STENCIL : K_STENCIL_SUMS, [&] { return launch_stencil_tma<float>(g, lat->st); });
+      StencilGroup<float> g;
+      if (!stencil_group_member(lat, in, out, write, reduce, scale, g)) return cudaErrorInvalidValue;
+      return launch(lat, kind, [&] { return launch_stencil<float>(g, lat->st); });
     }
-    StencilTmaGroup<double> g;
-    if (!stencil_group_member(lat, in, out, write, reduce, scale, g, true, zc)) return cudaErrorInvalidValue;
-    return launch(lat, write ? K_STENCIL : K_STENCIL_SUMS, [&] { return launch_stencil_tma<double>(g, lat->st); });
+    StencilGroup<double> g;
+    if (!stencil_group_member(lat, in, out, write, reduce, scale, g)) return cudaErrorInvalidValue;
+    return launch(lat, kind, [&] { return launch_stencil<double>(g, lat->st); });
   }
   // FFT terms: in place on `in` (out must equal in when writing); the scratch field is tmp.
   // A step on the live psi emits the next step's first pass and may skip its own.
@@ -892,9 +766,10 @@ static cudaError_t after_step(qf_lattice* lat, bool check, int nb, int snap_ever
 // Bookkeeping after a two-step pass (steps t and t+1): one buffer swap, two steps.
 static cudaError_t after_pair(qf_lattice* lat, int snap_every, cudaStream_t st) {
   if (lat->pending_scale) {
-    lat->K += lat->jcur - lat->K_check;  // (kcur is 0 whenever steps are paired)
+    lat->K += lat->jcur - lat->K_check;
     lat->renorm_step = lat->step;
   }
+  lat->K += 2 * lat->kcur;
   lat->pending_scale = false;
   lat->live = 1 - lat->live;
   lat->clean = true;
@@ -959,21 +834,15 @@ static cudaError_t run_chunk_graph(qf_lattice* lat, int check_every, int* flips)
   const int k = check_every - 1;
   const qf_lattice::Graph* hit = nullptr;
   for (auto& g : lat->graphs)
-    if (g.check_every == check_every && g.live == lat->live && g.tblock == lat->tblock &&
-        g.kzero == (lat->kcur == 0))
+    if (g.check_every == check_every && g.live == lat->live && g.tblock == lat->tblock)
       hit = &g;
   if (!hit) {
     // capture the k steps without touching the handle's state
     const int live0 = lat->live;
     const bool xv0 = lat->xfwd_valid, ps0 = lat->pending_scale, clean0 = lat->clean;
     const int64_t launches0 = lat->launches;
-    const bool pairs = lat->kinetic == QF_KIN_FDTD && lat->c64() && lat->tblock >= 2 && lat->tbmap_ok;
-    const int tzc = pairs ? tuned_tb_zchunk(lat) : 0;  // timed outside the capture
+    const bool pairs = lat->kinetic == QF_KIN_FDTD && lat->c64() && lat->tblock >= 2;
     tune_fft_tiles(lat);
-    if (lat->kinetic == QF_KIN_FDTD) {
-      if (lat->c64()) tuned_zchunk<float>(lat);
-      else tuned_zchunk<double>(lat);
-    }
     int nflip = 0;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(lat->st, cudaStreamCaptureModeThreadLocal);
@@ -982,7 +851,7 @@ static cudaError_t run_chunk_graph(qf_lattice* lat, int check_every, int* flips)
     for (int s = 0; s < k && e == cudaSuccess;) {
       const double* scale = lat->pending_scale ? &lat->sc()->scale[1] : &lat->sc()->scale[2];
       if (pairs && s + 2 <= k && fuse_pair(lat, t, check_every, check_every)) {
-        e = fdtd_pair(lat, scale, tzc);
+        e = fdtd_pair(lat, scale);
         s += 2;
         t += 2;
       } else {
@@ -1015,7 +884,7 @@ static cudaError_t run_chunk_graph(qf_lattice* lat, int check_every, int* flips)
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess) return e;
-    lat->graphs.push_back({check_every, live0, lat->tblock, lat->kcur == 0 ? 1 : 0, exec, nflip, nlaunch});
+    lat->graphs.push_back({check_every, live0, lat->tblock, exec, nflip, nlaunch});
     hit = &lat->graphs.back();
   }
   cudaError_t e = cudaGraphLaunch(hit->exec, lat->st);
@@ -1042,8 +911,7 @@ extern "C" qf_status qf_step_n(qf_lattice* lat, int64_t max_steps, double tol_ab
     const bool check = check_every > 0 && t % check_every == 0;
     const double* scale = lat->pending_scale ? &lat->sc()->scale[1] : &lat->sc()->scale[2];
     if (done + 2 <= max_steps && fuse_pair(lat, t, check_every, snap_every)) {
-      const int tzc = tuned_tb_zchunk(lat);
-      QF_CUDA(lat, fdtd_pair(lat, scale, tzc));
+      QF_CUDA(lat, fdtd_pair(lat, scale));
       QF_CUDA(lat, after_pair(lat, snap_every, lat->st));
       done += 2;
       continue;
@@ -1095,12 +963,8 @@ extern "C" qf_status qf_step_n(qf_lattice* lat, int64_t max_steps, double tol_ab
     }
   }
   if (steps_done) *steps_done = done;
-  // surface asynchronous launch failures and bounded-wait timeouts before reporting
+  // surface asynchronous launch failures before reporting (no kernel of a step waits on another)
   QF_CUDA(lat, cudaStreamSynchronize(lat->st));
-  if (lat->kinetic == QF_KIN_FDTD) {
-    qf_status s = check_device_error(lat);
-    if (s != QF_OK) return s;
-  }
   return status;
 }
 
@@ -1114,8 +978,6 @@ extern "C" qf_status qf_energies(qf_lattice* lat, qf_energy* out) {
 // <v|H|v>/<v|v> of a field into out (FP64 sums; the field is not modified).
 static qf_status measure(qf_lattice* lat, void* f, qf_energy* out) {
   int nb = 0;
-  if (lat->kinetic == QF_KIN_FDTD && f != lat->field(0) && f != lat->field(1) && !lat->fmap_ok)
-    return fail(lat, QF_ECUDA, "tensor map encoding unavailable");
   // FFT terms transform through tmp and read f; FDTD reads f only
   QF_CUDA(lat, kinetic_pass(lat, f, f, false, true, &lat->sc()->scale[0], &nb));
   QF_CUDA(lat, launch(lat, K_FINISH, [&] { return launch_finish(lat->partials(), nb, lat->sc(), 0, lat->st); }));
@@ -1549,7 +1411,7 @@ extern "C" qf_status qf_batch_members(qf_batch* b, int* count, int* status, int6
 // Whether a batch member's FDTD steps may run two per launch (the conditions of fuse_pair
 // that do not depend on the step's place in the check and snapshot schedule).
 static bool pairable(const qf_lattice* L) {
-  return L->kinetic == QF_KIN_FDTD && L->c64() && L->tblock >= 2 && L->clean && L->tbmap_ok && L->kcur == 0;
+  return L->kinetic == QF_KIN_FDTD && L->c64() && L->tblock >= 2 && L->clean;
 }
 
 // Issues the launches of one batch step for the running members `run` (check flags chk);
@@ -1592,7 +1454,7 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
       const int cnt = (int)std::min<size_t>(kGroupMax, g.size() - off);
       if (fdtd) {
         // single steps in one launch, pairs in one launch per kind of potential
-        StencilTmaGroup<float> sg;
+        StencilGroup<float> sg;
         StencilTbGroup tg[2];
         sg.count = 0;
         tg[0].count = tg[1].count = 0;
@@ -1604,22 +1466,20 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
           if (mode == 2) continue;
           if (mode == 1) {
             StencilTbGroup& t = tg[M->v_real ? 1 : 0];
-            tb_args(M, sq, tuned_tb_zchunk(M), t.m[t.count++]);
+            tb_args(M, sq, t.m[t.count++]);
             continue;
           }
-          const int zc = tuned_zchunk<float>(M);
-          if (!stencil_group_member<float>(M, M->psi(), M->tmp(), true, chk[q], sq, sg, sg.count == 0, zc))
-            return bfail(b, QF_ECUDA, "tensor map encoding failed");
-          // one error flag per launch: the first member's
-          nblk[q] = stencil_blocks<float>(M->d.n, zc);
+          if (!stencil_group_member<float>(M, M->psi(), M->tmp(), true, chk[q], sq, sg, sg.count == 0))
+            return bfail(b, QF_EINVAL, "too many members in a group");
+          nblk[q] = stencil_blocks(M->d.n);
         }
         if (sg.count > 0) {
-          QF_BCUDA(b, launch_stencil_tma<float>(sg, st));
+          QF_BCUDA(b, launch_stencil<float>(sg, st));
           b->launches += 1;
         }
         for (auto& t : tg)
           if (t.count > 0) {
-            QF_BCUDA(b, launch_stencil_tb_group(t, st));
+            QF_BCUDA(b, launch_stencil_tb(t, st));
             b->launches += 1;
           }
       } else {
@@ -1687,7 +1547,6 @@ static qf_status batch_chunk_graph(qf_batch* b, const std::vector<int>& run, int
   for (size_t q = 0; q < run.size(); ++q) {
     qf_lattice* L = b->m[run[q]].lat;
     pair[q] = pairable(L) ? 1 : 0;
-    if (pair[q]) tuned_tb_zchunk(L);  // timed outside the capture
   }
   const qf_batch::BGraph* hit = nullptr;
   for (auto& g : b->graphs)
@@ -1876,11 +1735,6 @@ extern "C" qf_status qf_batch_step(qf_batch* b, int64_t steps, int check_every, 
     }
   }
   QF_BCUDA(b, cudaStreamSynchronize(st));
-  for (auto& x : b->m)
-    if (x.lat->kinetic == QF_KIN_FDTD) {
-      qf_status es = check_device_error(x.lat);
-      if (es != QF_OK) return bfail(b, es, x.lat->err);
-    }
   int nr = 0;
   for (auto& x : b->m) {
     if (x.status == QF_BATCH_RUNNING && x.steps_done >= x.max_steps) x.status = QF_ENOTCONV;

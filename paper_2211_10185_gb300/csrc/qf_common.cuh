@@ -274,8 +274,8 @@ bool set_fft_tile_choice(int n, int v);
 // Whether the FFT path has kernels for this n.
 bool fft_supported(int n);
 
-template <typename R>
-int stencil_blocks(int n, int zc = 0);
+// Partial-sum rows of the FDTD step for lattice size n.
+int stencil_blocks(int n);
 
 // Finishing reduction: sums nblocks partial rows in index order into sc->sums, then the
 // energy; with set_scale also the step scales sc->scale[1..2] and their exponents k, j in

@@ -1,259 +1,253 @@
-// Temporally blocked FDTD steps: two imaginary-time steps with the kinetic term of Eq.
-// HK0 per pass over HBM (complex FP32 fields), sm_103a.
+// Two FDTD steps per pass over HBM (kinetic term of Eq. HK0, complex FP32 fields), sm_103a.
 //
 // Two consecutive steps read psi_t and V and write psi_{t+2}; the intermediate psi_{t+1}
-// lives only in shared memory.  A block owns a 32 x 32 column tile of the output and
-// marches through a chunk of z (chunk sizes differ by at most one plane, so the number of
-// chunks can be chosen to fill whole waves of resident blocks).  Three levels are in flight at once:
-//   level 0  psi_t on the tile plus a halo of 2 (36 x 36), streamed plane by plane with
-//            cp.async.bulk.tensor into a ring of six buffers (each with an mbarrier);
-//   level 1  psi_{t+1} on the tile plus a halo of 1 (34 x 34), computed one plane behind
-//            level 0 into a ring of four buffers;
-//   level 2  psi_{t+2} on the tile, computed two planes behind level 1 and stored.
-// One block barrier per plane separates the levels: level 1 of plane p needs level-0
-// planes p-1..p+1, level 2 of plane p needs level-1 planes p-1..p+1, and the ring slots
-// written in an iteration are never the ones read in it.
+// never leaves the registers of a warp.  A warp owns 4 rows of 28 output columns and marches
+// through a chunk of z, lane = x (32 columns: the outputs and a halo of 2 on either side).
+// Three levels are in flight at once:
+//   level 0  psi_t on 8 rows (halo 2), three planes of it in registers;
+//   level 1  psi_{t+1} on 6 rows (halo 1) of the middle plane: y- and z-neighbours are the
+//            lane's own registers, x-neighbours come by shuffle;
+//   level 2  psi_{t+2} on the 4 rows, one plane behind level 1, stored by lanes 2 .. 29.
+// Loads of the plane after next are issued once level 1 has freed the oldest plane's
+// registers.  No shared memory and no barrier, one warp per block (so that everything but
+// the column is the same in all lanes for the compiler; blocks of 4 or 8 warps, whose halo
+// rows meet in L1, came out 15-35 % slower).  The arithmetic is on packed pairs (re, im), one
+// instruction where two were needed, and the lane's address of a row is one instruction.
+//
+// What bounds it: instruction issue and load latency about equally (N = 256: 61 M warp
+// instructions, 56 % of issue slots, 16 warps per SM at 128 registers), not yet HBM (20
+// bytes per site and two steps).  The form before kept both levels in shared memory
+// (TMA-filled 36 x 36 planes, seven reads a site, a block barrier per plane, about 190
+// instructions a site).  Two steps, before and now: N = 64: 31 / 10 us, 128: 25 / 18 us,
+// 250: 131 / 83 us (3.7 TB/s of the 20 bytes), 256: 134 / 95 us, 384: 402 / 259 us.
 //
 // Sites with an index 0 (the Dirichlet planes) and sites outside the lattice are zero at
 // every level; the input field must already be zero on the Dirichlet planes (true after
-// any FDTD step).  Each site is computed with the same rounded operations as the
-// single-step kernel, so two single steps and one blocked pass give the same bits.
+// any FDTD step), so a load from outside is redirected to one of them.  Each site is computed
+// with the same rounded operations as the single-step kernel, so two single steps and one
+// pass give the same bits.
 //
-// Every wait is bounded as in the single-step kernel: on time-out the block records a
-// flag, drains its own copies with a bounded wait and returns.
-//
-// A group launch (stencil_tb_group_kernel) steps several lattices of any sizes at once:
-// a one-dimensional grid whose blocks are numbered member by member from a block table,
-// each block running the same body on its member's tile and z-chunk.
+// A group launch steps several lattices of any sizes at once: a one-dimensional grid whose
+// blocks are numbered member by member from a block table; a lone lattice is a group of one.
 #pragma once
-#include "qf_stencil_tma.cuh"
+#include <type_traits>
+#include <utility>
+
+#include "qf_stencil_flat.cuh"
 
 namespace qf {
 
-constexpr int TB_X = 32, TB_Y = 32, TB_ROWS = 4;
-constexpr int TB_THREADS = TB_X * (TB_Y / TB_ROWS);  // 256
-constexpr int TB_W0 = TB_X + 4, TB_H0 = TB_Y + 4;    // level-0 box: halo 2
-constexpr int TB_W1 = TB_X + 2, TB_H1 = TB_Y + 2;    // level-1 region: halo 1
-constexpr int TB_D0 = 6, TB_D1 = 4;                  // ring depths
-constexpr int TB_L0_WORDS = TB_W0 * TB_H0;           // 1296 complex = 10368 B (81 x 128 B)
-constexpr int TB_L1_SITES = TB_W1 * TB_H1;           // 1156
-constexpr int TB_L1_STRIDE = (TB_L1_SITES + 15) / 16 * 16;
-constexpr int TB_L1_PER_THREAD = (TB_L1_SITES + TB_THREADS - 1) / TB_THREADS;  // 5
-constexpr unsigned TB_L0_BYTES = TB_L0_WORDS * 8u;
+constexpr int TB_XOUT = 28, TB_ROWS = 4;
+constexpr int TB_R0 = TB_ROWS + 4, TB_R1 = TB_ROWS + 2;
 
-struct alignas(64) StencilTbArgs {
-  CUtensorMap map;        // input field psi_t, box TB_W0 x TB_H0 x 1 of 8-byte elements
+struct StencilTbArgs {
+  const cpx<float>* in;   // psi_t
   cpx<float>* out;        // psi_{t+2}
   const void* v;          // V: float (v_real) or complex float
   int v_real;
   float half_dtau;        // dtau / 2
   float kd;               // dtau / (2 m a^2)
-  const double* scale;    // renormalisation applied in the first of the two steps
+  const double* scale;    // output scale of the first of the two steps
+  const double* scale2;   // output scale of the second
   int n;
-  int nzb;                // z-chunks per column tile: chunk b holds planes [b n/nzb, (b+1) n/nzb)
-  int* err;               // set to 1 when a bounded wait ran out
+  int nzb;                // z-chunks: chunk b holds planes [b n/nzb, (b+1) n/nzb)
 };
 
-constexpr size_t stencil_tb_smem() { return (size_t)(TB_D0 * TB_L0_WORDS + TB_D1 * TB_L1_STRIDE) * 8; }
-
-__device__ __forceinline__ void tb_plane(const CUtensorMap* map, unsigned long long* bar, void* dst, int x0, int y0,
-                                         int z) {
-  mbar_expect_tx(bar, TB_L0_BYTES);
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(
-          smem_u32(dst)),
-      "l"(map), "r"(x0 - 2), "r"(y0 - 2), "r"(z), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// V at offset `off` of plane p (the plane's base address computed once per plane)
-template <bool VREAL>
-__device__ __forceinline__ cpx<float> tb_v(const StencilTbArgs& g, long long plane_off, int off) {
-  if constexpr (VREAL) return mk<float>((reinterpret_cast<const float*>(g.v) + plane_off)[off], 0.f);
-  else return (reinterpret_cast<const cpx<float>*>(g.v) + plane_off)[off];
-}
-
 // Members of a group launch: blocks of member i are start[i] .. start[i+1] - 1 (the
-// launcher fills start), each member (n/32)^2 nzb blocks.  All members have the same kind
-// of potential (v_real).
+// launcher fills start).  All members have the same kind of potential (v_real).
 struct StencilTbGroup {
   StencilTbArgs m[kGroupMax];
   int start[kGroupMax + 1];
   int count;
 };
 
+__host__ __device__ inline int stencil_tb_xtiles(int n) { return (n + TB_XOUT - 1) / TB_XOUT; }
+__host__ __device__ inline int stencil_tb_ytiles(int n) { return (n + TB_ROWS - 1) / TB_ROWS; }
 __host__ __device__ inline int stencil_tb_member_blocks(int n, int nzb) {
-  return ((n + TB_X - 1) / TB_X) * ((n + TB_Y - 1) / TB_Y) * nzb;
+  return stencil_tb_xtiles(n) * stencil_tb_ytiles(n) * nzb;
 }
 
-// The two steps for column tile (bx, by) and z-chunk bz of the lattice in g.  VREAL: the
-// potential is real (g.v holds floats).  g must live in kernel parameter space (its
-// tensor map is read by the copies).
-template <bool VREAL>
-__device__ __forceinline__ void stencil_tb_body(const StencilTbArgs& g, int bx, int by, int bz) {
-  extern __shared__ __align__(128) unsigned long long tb_dyn[];
-  cpx<float>* l0 = reinterpret_cast<cpx<float>*>(tb_dyn);
-  cpx<float>* l1 = l0 + TB_D0 * TB_L0_WORDS;
-  __shared__ alignas(8) unsigned long long bars[TB_D0];
-  const int n = g.n;
-  const long long plane_sites = (long long)n * n;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  const int x0 = bx * TB_X, y0 = by * TB_Y;
-  const int z0 = (int)((long long)bz * n / g.nzb), z1 = (int)((long long)(bz + 1) * n / g.nzb);
-  const int pbase = z0 - 2, last0 = z1 + 1;  // level-0 planes z0-2 .. z1+1
-  const float hd = g.half_dtau, kd = g.kd;
-  const float sc1 = (float)*g.scale;
+// z-chunks for lattice size n.  Two planes a chunk while all warps fit the GPU at once (16
+// resident warps per SM at 128 registers): a small lattice is bound by the latency of a
+// warp's march.  Beyond that as many chunks as make whole waves of resident warps, with at
+// least 16 planes each (a chunk repeats two planes of level 1 and four loads); one wave if
+// its chunks are shorter than that.  Measured, us per pass: N = 64: 12 (2-4 planes), 28 (16);
+// N = 192: 67 in one wave, 84 in 1.1; N = 250: 135 / 135 / 132 / 136 in 1 / 2 / 3 / 4 waves;
+// N = 384: 440 (3 waves), 401 (13), 430 (26).
+inline int stencil_tb_chunks(int n) {
+  const long long cap = 152 * 16, tiles = stencil_tb_member_blocks(n, 1);
+  if (tiles * ((n + 1) / 2) <= cap) return (n + 1) / 2;
+  long long best = cap / tiles > 1 ? cap / tiles : 1;
+  for (long long w = 2; w * cap / tiles * 16 <= n; ++w) best = w * cap / tiles > 1 ? w * cap / tiles : 1;
+  return (int)best;
+}
 
-  // level-1 sites of this thread: flat index i = tid + 256 q over the 34 x 34 region
-  int o0[TB_L1_PER_THREAD], o1[TB_L1_PER_THREAD], gs[TB_L1_PER_THREAD];
-  bool in1[TB_L1_PER_THREAD], has1[TB_L1_PER_THREAD];
-#pragma unroll
-  for (int q = 0; q < TB_L1_PER_THREAD; ++q) {
-    const int i = tid + TB_THREADS * q;
-    const int ly = i / TB_W1, lx = i - ly * TB_W1;
-    const int x = x0 - 1 + lx, y = y0 - 1 + ly;
-    has1[q] = i < TB_L1_SITES;
-    in1[q] = has1[q] && x >= 1 && x < n && y >= 1 && y < n;
-    o0[q] = (ly + 1) * TB_W0 + lx + 1;
-    o1[q] = ly * TB_W1 + lx;
-    gs[q] = in1[q] ? y * n + x : 0;
+// ---- packed complex FP32 (re in the low half): each half rounded as the scalar operation ---
+using pk = unsigned long long;
+__device__ __forceinline__ pk pk_make(float lo, float hi) {
+  pk r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ cpx<float> pk_get(pk a) {
+  cpx<float> c;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(a));
+  return c;
+}
+__device__ __forceinline__ pk pk_add(pk a, pk b) {
+  pk r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ pk pk_mul(pk a, pk b) {
+  pk r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ pk pk_fma(pk a, pk b, pk c) {
+  pk r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// base + k * stride bytes in one instruction (k a constant, stride the same in all lanes)
+template <int K>
+__device__ __forceinline__ unsigned long long tb_addr(unsigned long long base, unsigned stride) {
+  unsigned long long r;
+  if constexpr (K == 0) r = base;
+  else asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(stride), "n"(K), "l"(base));
+  return r;
+}
+template <typename F, int... I>
+__device__ __forceinline__ void tb_rows(F&& f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+
+// One site: c and its neighbours, potential (vx, vy), output scale sc; live: whether the site
+// may be nonzero (else the result is a zero times the numerator).  The same operations, in
+// the same order, as fdtd_update after lap_of(six_sum).
+template <bool VREAL>
+__device__ __forceinline__ pk tb_site(pk c, pk xm, pk xp, pk ym, pk yp, pk zm, pk zp, float vx, float vy, float hd,
+                                      pk kd2, pk m6, float sc, bool live) {
+  const pk nbs = pk_add(pk_add(pk_add(xm, xp), pk_add(ym, yp)), pk_add(zm, zp));
+  const pk lap = pk_fma(m6, c, nbs);
+  const float dx = fma_rn<float>(hd, vx, 1.f), tx = add_rn<float>(2.f, -dx);
+  if constexpr (VREAL) {
+    const float inv = live ? scaled_inverse<float>(sc, dx) : 0.f;
+    return pk_mul(pk_fma(kd2, lap, pk_mul(pk_make(tx, tx), c)), pk_make(inv, inv));
+  } else {
+    // (2 - d) psi = (tx - i dy) psi, d = dx + i dy
+    const float dy = mul_rn<float>(hd, vy);
+    const cpx<float> cc = pk_get(c);
+    const float ax = fma_rn<float>(tx, cc.x, mul_rn<float>(dy, cc.y));
+    const float ay = fma_rn<float>(tx, cc.y, -mul_rn<float>(dy, cc.x));
+    const cpx<float> nn = pk_get(pk_fma(kd2, lap, pk_make(ax, ay)));
+    const float inv = live ? scaled_inverse<float>(sc, fma_rn<float>(dx, dx, mul_rn<float>(dy, dy))) : 0.f;
+    return pk_make(mul_rn<float>(fma_rn<float>(nn.x, dx, mul_rn<float>(nn.y, dy)), inv),
+                   mul_rn<float>(fma_rn<float>(nn.y, dx, -mul_rn<float>(nn.x, dy)), inv));
   }
-  // output sites: column x0 + tx, rows y0 + 4 ty .. y0 + 4 ty + 3
-  const int ox = x0 + tx, oy = y0 + TB_ROWS * ty;
-  bool in2[TB_ROWS], st2[TB_ROWS];
-#pragma unroll
-  for (int k = 0; k < TB_ROWS; ++k) {
-    st2[k] = ox < n && oy + k < n;
-    in2[k] = st2[k] && ox >= 1 && oy + k >= 1;
-  }
-  const int o2 = oy * n + ox;  // in-plane offset of this thread's first output row
-  auto load_v1 = [&](int p, cpx<float>(&v)[TB_L1_PER_THREAD]) {
-    const bool zin = p >= 1 && p < n;
-    const long long po = zin ? p * plane_sites : 0;
-#pragma unroll
-    for (int q = 0; q < TB_L1_PER_THREAD; ++q)
-      v[q] = (zin && in1[q]) ? tb_v<VREAL>(g, po, gs[q]) : mk<float>(0.f, 0.f);
+}
+
+// The two steps for output columns [28 bx, 28 bx + 28), rows [y0, y0 + 4) and planes [z0, z1)
+// of the lattice in g.  EDGE: some row of the warp's levels is row 0 or lies outside the
+// lattice.  Positions that must read as zero are redirected to plane 0 or column 0 (zero);
+// a dead position next to one that holds a non-finite value is zero in the output all the
+// same (selected), and its level-1 value only reaches positions that are non-finite already.
+template <bool VREAL, bool EDGE, bool PRE>
+__device__ __forceinline__ void stencil_tb_march(const StencilTbArgs& g, int bx, int y0, int z0, int z1) {
+  using u64 = unsigned long long;
+  const int n = g.n, lane = threadIdx.x;
+  const long long n2 = (long long)n * n;
+  const int x = bx * TB_XOUT - 2 + lane;
+  const bool xlive = x >= 1 && x < n;
+  const bool xout = lane >= 2 && lane < 2 + TB_XOUT && x < n;
+  const unsigned xo = xlive ? x : 0;  // column 0 is zero
+  const float sc1 = (float)*g.scale, sc2 = (float)*g.scale2, hd = g.half_dtau;
+  const pk kd2 = pk_make(g.kd, g.kd), m6 = pk_make(-6.f, -6.f);
+  const unsigned s8 = n * 8, sv = n * (VREAL ? 4 : 8);
+  const u64 in0 = (u64)(reinterpret_cast<const pk*>(g.in) + xo), out0 = (u64)(reinterpret_cast<pk*>(g.out) + x);
+  const u64 v0 = VREAL ? (u64)(reinterpret_cast<const float*>(g.v) + xo) : (u64)(reinterpret_cast<const pk*>(g.v) + xo);
+  auto ylive = [&](int y) { return !EDGE || (y >= 1 && y < n); };
+  // row i of level 0 is y0 - 2 + i
+  auto zlo = [&](int z) { return (EDGE ? 0LL : (long long)(y0 - 2) * n) + (z >= 1 && z < n ? z * n2 : 0LL); };
+  auto erow = [&](int i) { return ylive(y0 - 2 + i) ? (unsigned)(y0 - 2 + i) : 0u; };
+  using R0 = std::make_integer_sequence<int, TB_R0>;
+  using R1 = std::make_integer_sequence<int, TB_R1>;
+  pk A[3][TB_R0], B[3][TB_R1];
+  float vx[3][TB_R1], vy[VREAL ? 1 : 3][VREAL ? 1 : TB_R1];
+  auto load0 = [&](pk(&a)[TB_R0], int z) {
+    const u64 q = in0 + 8 * zlo(z);
+    tb_rows([&](auto i) {
+      const u64 p = EDGE ? q + (u64)erow(i) * s8 : tb_addr<i()>(q, s8);
+      asm volatile("ld.global.nc.b64 %0, [%1];" : "=l"(a[i()]) : "l"(p));
+    }, R0{});
   };
-  auto load_v2 = [&](int p, cpx<float>(&v)[TB_ROWS]) {
-    const bool zin = p >= 1 && p < n;
-    const long long po = zin ? p * plane_sites : 0;
-#pragma unroll
-    for (int k = 0; k < TB_ROWS; ++k)
-      v[k] = (zin && in2[k]) ? tb_v<VREAL>(g, po, o2 + k * n) : mk<float>(0.f, 0.f);
+  auto loadv = [&](auto kc, int z) {
+    constexpr int K = decltype(kc)::value;
+    const u64 q = v0 + (VREAL ? 4 : 8) * zlo(z);
+    tb_rows([&](auto i) {
+      const u64 p = EDGE ? q + (u64)erow(i + 1) * sv : tb_addr<i() + 1>(q, sv);
+      if constexpr (VREAL) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(vx[K][i()]) : "l"(p));
+      else asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(vx[K][i()]), "=f"(vy[VREAL ? 0 : K][VREAL ? 0 : i()]) : "l"(p));
+    }, R1{});
   };
-
-  if (tid == 0) {
-    for (int b = 0; b < TB_D0; ++b) mbar_init(&bars[b], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  __syncthreads();
-  int issued = pbase - 1;
-  if (tid == 0)
-    for (int p = pbase; p <= last0 && p < pbase + TB_D0; ++p) {
-      tb_plane(&g.map, &bars[p - pbase], l0 + (p - pbase) * TB_L0_WORDS, x0, y0, p);
-      issued = p;
-    }
-  cpx<float> v1n[TB_L1_PER_THREAD], v2n[TB_ROWS];
-  load_v1(z0 - 1, v1n);
-  load_v2(z0 - 2, v2n);
-  int waited = pbase - 1;
-  bool ok = true;
-  for (int j = z0; j <= z1 + 2; ++j) {
-    cpx<float> v1c[TB_L1_PER_THREAD], v2c[TB_ROWS];
+  // PRE: prefetch into L2 of the warp's own rows, TB_AHEAD planes on, one line a lane: lanes
+  // 0-11 take psi (3 lines of 128 bytes cover 32 sites of a row), lanes 12-19 V
+  constexpr int TB_AHEAD = 4;
+  const int pl = lane < 12 ? lane : lane - 12, prow = min(y0 + (lane < 12 ? pl / 3 : pl >> 1), n - 1);
+  const int pcol = min(max(bx * TB_XOUT - 2, 0) + (lane < 12 ? (pl % 3) * 16 : (pl & 1) * (VREAL ? 32 : 16)), n - 1);
+  const u64 pre0 = lane < 12 ? (u64)(reinterpret_cast<const pk*>(g.in) + (long long)prow * n + pcol)
+                             : (u64)g.v + (VREAL ? 4 : 8) * ((long long)prow * n + pcol);
+  const u64 pst = (u64)n2 * (lane < 12 || !VREAL ? 8 : 4);
+  // psi_{t+1} of plane p into B[K]: level-0 planes p-1, p, p+1 in A[K], A[K+1], A[K+2] (mod 3)
+  // and V of planes p-1, p in v[K+2], v[K]; then psi_{t+2} of plane p-1 from B[K+1], B[K+2], B[K]
+  auto plane = [&](auto kc, int p) {
+    constexpr int K = decltype(kc)::value, K1 = (K + 1) % 3, K2 = (K + 2) % 3;
+    if (p < z1) loadv(std::integral_constant<int, K1>{}, p + 1);
+    if constexpr (PRE)
+      if (lane < 20 && p + TB_AHEAD < n)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(pre0 + (u64)(p + TB_AHEAD) * pst));
+    const bool live1 = xlive && p >= 1 && p < n;
 #pragma unroll
-    for (int q = 0; q < TB_L1_PER_THREAD; ++q) v1c[q] = v1n[q];
-#pragma unroll
-    for (int k = 0; k < TB_ROWS; ++k) v2c[k] = v2n[k];
-    if (j <= z1) load_v1(j, v1n);       // level-1 plane of the next iteration
-    if (j - 2 >= z0) load_v2(j - 2, v2n);  // level-2 plane of the next iteration
-    // level-0 planes up to j must have landed: thread 0 polls (bounded), the block learns
-    // the outcome at the barrier, then every thread observes the completed phases itself
-    const int need = min(j, last0);
-    bool mine = true;
-    if (tid == 0)
-      while (waited < need && mine) {
-        const int u = waited + 1 - pbase;
-        mine = mbar_wait_bounded(&bars[u % TB_D0], (unsigned)((u / TB_D0) & 1));
-        if (mine) ++waited;
-      }
-    ok = __syncthreads_and(mine) != 0;
-    if (!ok) break;
-    if (tid != 0)
-      for (; waited < need; ++waited) {
-        const int u = waited + 1 - pbase;
-        mbar_try_wait(&bars[u % TB_D0], (unsigned)((u / TB_D0) & 1));  // completed: returns at once
-      }
-    // the slot of level-0 plane j-3 was last read in the previous iteration
-    if (tid == 0 && issued < last0 && issued + 1 <= j + 3) {
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      const int p = issued + 1;
-      tb_plane(&g.map, &bars[(p - pbase) % TB_D0], l0 + ((p - pbase) % TB_D0) * TB_L0_WORDS, x0, y0, p);
-      issued = p;
+    for (int i = 0; i < TB_R1; ++i) {
+      const pk c = A[K1][i + 1];
+      const pk xm = __shfl_up_sync(0xffffffffu, c, 1), xp = __shfl_down_sync(0xffffffffu, c, 1);
+      B[K][i] = tb_site<VREAL>(c, xm, xp, A[K1][i], A[K1][i + 2], A[K][i + 1], A[K2][i + 1], vx[K][i],
+                               VREAL ? 0.f : vy[VREAL ? 0 : K][VREAL ? 0 : i], hd, kd2, m6, sc1,
+                               live1 && ylive(y0 - 1 + i));
     }
-    // level 1: psi_{t+1} on plane j-1 (halo 1)
-    if (j - 1 <= z1) {
-      const int p = j - 1;
-      const bool zin = p >= 1 && p < n;
-      const cpx<float>* am = l0 + ((p - 1 - pbase) % TB_D0) * TB_L0_WORDS;
-      const cpx<float>* ac = l0 + ((p - pbase) % TB_D0) * TB_L0_WORDS;
-      const cpx<float>* ap = l0 + ((p + 1 - pbase) % TB_D0) * TB_L0_WORDS;
-      cpx<float>* w = l1 + ((p - (z0 - 1)) % TB_D1) * TB_L1_STRIDE;
-      // branch-free: every position is computed (halo and wall positions read zeros or
-      // finite values) and the Dirichlet/outside ones are replaced by 0; only the last
-      // round of the flat index is partial
-#pragma unroll
-      for (int q = 0; q < TB_L1_PER_THREAD; ++q) {
-        if (q == TB_L1_PER_THREAD - 1 && !has1[q]) break;
-        const int o = o0[q];
-        const cpx<float> c = ac[o];
-        const cpx<float> lap =
-            lap_of<float>(c, six_sum<float>(ac[o - 1], ac[o + 1], ac[o - TB_W0], ac[o + TB_W0], am[o], ap[o]));
-        const cpx<float> u = fdtd_update<float>(c, lap, v1c[q], VREAL, hd, kd, sc1);
-        const bool live = zin && in1[q];
-        w[o1[q]] = mk<float>(live ? u.x : 0.f, live ? u.y : 0.f);
-      }
+    if (p < z1) load0(A[K], p + 2);
+    if (p > z0) {
+      const int q = p - 1;
+      const u64 dst = out0 + 8 * (q * n2 + (long long)y0 * n);
+      tb_rows([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        const pk c = B[K2][i + 1];
+        const pk xm = __shfl_up_sync(0xffffffffu, c, 1), xp = __shfl_down_sync(0xffffffffu, c, 1);
+        const pk u = tb_site<VREAL>(c, xm, xp, B[K2][i], B[K2][i + 2], B[K1][i + 1], B[K][i + 1], vx[K2][i + 1],
+                                    VREAL ? 0.f : vy[VREAL ? 0 : K2][VREAL ? 0 : i + 1], hd, kd2, m6, sc2, true);
+        const pk o = xlive && q >= 1 && ylive(y0 + i) ? u : 0ull;
+        const int st = xout && (!EDGE || y0 + i < n);
+        asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %2, 0;\n @p st.global.b64 [%0], %1;\n}\n" ::"l"(
+                         tb_addr<i>(dst, s8)), "l"(o), "r"(st) : "memory");
+      }, std::make_integer_sequence<int, TB_ROWS>{});
     }
-    // level 2: psi_{t+2} on plane j-3 (the tile), stored
-    if (j - 3 >= z0) {
-      const int p = j - 3;
-      const bool zin = p >= 1 && p < n;
-      const cpx<float>* bm = l1 + ((p - 1 - (z0 - 1)) % TB_D1) * TB_L1_STRIDE;
-      const cpx<float>* bc = l1 + ((p - (z0 - 1)) % TB_D1) * TB_L1_STRIDE;
-      const cpx<float>* bp = l1 + ((p + 1 - (z0 - 1)) % TB_D1) * TB_L1_STRIDE;
-      // column of the centre plane: local rows 4 ty .. 4 ty + 5 (level-1 coordinates)
-      const int base = (TB_ROWS * ty) * TB_W1 + tx + 1;
-      cpx<float> col[TB_ROWS + 2];
-#pragma unroll
-      for (int k = 0; k < TB_ROWS + 2; ++k) col[k] = bc[base + k * TB_W1];
-      cpx<float>* dst = g.out + (p * (long long)n + oy) * n + ox;
-#pragma unroll
-      for (int k = 0; k < TB_ROWS; ++k) {
-        const int o = base + (k + 1) * TB_W1;
-        const cpx<float> c = col[k + 1];
-        const cpx<float> lap = lap_of<float>(c, six_sum<float>(bc[o - 1], bc[o + 1], col[k], col[k + 2], bm[o], bp[o]));
-        const cpx<float> u = fdtd_update<float>(c, lap, v2c[k], VREAL, hd, kd, 1.0f);
-        const bool live = zin && in2[k];
-        if (st2[k]) dst[(long long)k * n] = mk<float>(live ? u.x : 0.f, live ? u.y : 0.f);
-      }
-    }
-  }
-  if (!ok && tid == 0) {
-    atomicExch(g.err, 1);
-    // copies already issued may still land in this block's shared memory
-    for (int p = waited + 1; p <= issued; ++p) {
-      const int u = p - pbase;
-      mbar_wait_bounded(&bars[u % TB_D0], (unsigned)((u / TB_D0) & 1));
-    }
+  };
+  load0(A[0], z0 - 2);
+  load0(A[1], z0 - 1);
+  load0(A[2], z0);
+  loadv(std::integral_constant<int, 0>{}, z0 - 1);
+  for (int p = z0 - 1; p <= z1; p += 3) {
+    plane(std::integral_constant<int, 0>{}, p);
+    if (p + 1 > z1) break;
+    plane(std::integral_constant<int, 1>{}, p + 1);
+    if (p + 2 > z1) break;
+    plane(std::integral_constant<int, 2>{}, p + 2);
   }
 }
 
-template <bool VREAL>
-__global__ void __launch_bounds__(TB_THREADS, 2) stencil_tb_kernel(const __grid_constant__ StencilTbArgs g) {
-  stencil_tb_body<VREAL>(g, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-
-template <bool VREAL>
-__global__ void __launch_bounds__(TB_THREADS, 2) stencil_tb_group_kernel(const __grid_constant__ StencilTbGroup gr) {
+template <bool VREAL, bool PRE>
+__global__ void __launch_bounds__(32, VREAL ? 16 : 12) stencil_tb_kernel(const __grid_constant__ StencilTbGroup gr) {
   // member of this block: the last i with start[i] <= block
   int member = 0;
   {
@@ -265,9 +259,14 @@ __global__ void __launch_bounds__(TB_THREADS, 2) stencil_tb_group_kernel(const _
     }
   }
   const StencilTbArgs& g = gr.m[member];
-  const int nbx = (g.n + TB_X - 1) / TB_X, nby = (g.n + TB_Y - 1) / TB_Y;
+  const int nbx = stencil_tb_xtiles(g.n), nby = stencil_tb_ytiles(g.n);
   const int local = (int)blockIdx.x - gr.start[member];
-  stencil_tb_body<VREAL>(g, local % nbx, (local / nbx) % nby, local / (nbx * nby));
+  const int bx = local % nbx, by = (local / nbx) % nby, bz = local / (nbx * nby);
+  const int y0 = by * TB_ROWS;
+  const int z0 = (int)((long long)bz * g.n / g.nzb), z1 = (int)((long long)(bz + 1) * g.n / g.nzb);
+  const bool inner = y0 >= 2 && y0 + TB_ROWS + 2 <= g.n;
+  if (inner) stencil_tb_march<VREAL, false, PRE>(g, bx, y0, z0, z1);
+  else stencil_tb_march<VREAL, true, PRE>(g, bx, y0, z0, z1);
 }
 
 }  // namespace qf
