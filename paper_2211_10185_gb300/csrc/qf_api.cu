@@ -18,6 +18,7 @@
 
 #include "../../include/qfdtd.h"
 #include "qf_common.cuh"
+#include "qf_fft_res.cuh"
 #include "qf_stencil_tb.cuh"
 
 namespace qf {
@@ -45,14 +46,14 @@ static size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 enum KernelKind {
   K_FFT_X_FWD = 0, K_FFT_Y_FWD, K_FFT_Z_MID, K_FFT_Y_INV, K_FFT_X_INV_UPDATE, K_STENCIL, K_FINISH, K_GS_DOTS,
   K_GS_AXPY, K_SCALE_COPY, K_PARITY, K_CONVERT, K_FFT_X_INV_SUMS, K_STENCIL_SUMS, K_STENCIL_2STEP, K_FFT2_XY_FWD,
-  K_FFT2_YZ_MID, K_FFT2_XY_INV_UPDATE, K_FFT2_XY_INV_SUMS, K_FFT2_XY_FWD_SUMS, K_FFT2_YZ_SUMS, K_NUM_KINDS
+  K_FFT2_YZ_MID, K_FFT2_XY_INV_UPDATE, K_FFT2_XY_INV_SUMS, K_FFT2_XY_FWD_SUMS, K_FFT2_YZ_SUMS, K_FFT_RES, K_NUM_KINDS
 };
 static const char* kKindNames[K_NUM_KINDS] = {"fft_x_fwd", "fft_y_fwd", "fft_z_mid_T", "fft_y_inv",
                                                "fft_x_inv_update", "stencil_step", "finish_sums", "gs_dots",
                                                "gs_axpy", "scale_copy", "parity", "convert", "fft_x_inv_sums",
                                                "stencil_sums", "stencil_2step", "fft2_xy_fwd", "fft2_yz_mid_T",
                                                "fft2_xy_inv_update", "fft2_xy_inv_sums", "fft2_xy_fwd_sums",
-                                               "fft2_yz_sums"};
+                                               "fft2_yz_sums", "fft_resident_steps"};
 static const int kEventPool = 4096;
 
 struct Layout {
@@ -193,6 +194,12 @@ struct qf_lattice {
 // The FFT step of this lattice runs the two-pass kernels.
 static bool uses_fft2(const qf_lattice* lat) {
   return lat->two_pass && lat->c64() && lat->kinetic != QF_KIN_FDTD && fft2_supported(lat->d.n);
+}
+
+// The FFT step of this lattice runs the resident kernel (many steps per launch).
+static bool uses_res(const qf_lattice* lat) {
+  return lat->two_pass && lat->c64() && lat->kinetic > QF_KIN_FDTD && res_supported(lat->d.n) &&
+         fft_res_blocks(lat->d.n) > 0;
 }
 
 static void drop_graphs(qf_lattice* lat) {
@@ -531,6 +538,26 @@ static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduc
   return p;
 }
 
+// Arguments of nsteps resident steps on the live psi.
+static ResArgs res_args(qf_lattice* lat, const double* scale, int nsteps) {
+  const FftPassArgs<float> p = fft_args<float>(lat, lat->psi(), true, false, scale);
+  ResArgs r{};
+  r.psi = p.psi;
+  r.v = p.v;
+  r.symbol = p.symbol;
+  r.scale = scale;
+  r.scale2 = &lat->sc()->scale[2];
+  r.partials = p.partials;
+  r.tcoef = p.tcoef;
+  r.am2 = p.am2;
+  r.half_dtau = p.half_dtau;
+  r.dtau = p.dtau;
+  r.err = &lat->sc()->err[0];
+  r.kinetic = p.kinetic;
+  r.nsteps = nsteps;
+  return r;
+}
+
 template <typename R>
 static StencilArgs<R> stencil_args(qf_lattice* lat, void* in, void* out, bool write, bool reduce,
                                    const double* scale) {
@@ -608,6 +635,18 @@ static void tune_fft_tiles(qf_lattice* lat) {
   lat->xfwd_valid = false;  // the scratch field was overwritten
 }
 
+// Reads and clears the bounded-wait failure flag of a lattice (resident FFT steps).
+static qf_status check_device_error(qf_lattice* lat) {
+  int err = 0;
+  QF_CUDA(lat, cudaMemcpyAsync(&err, &lat->sc()->err[0], sizeof(int), cudaMemcpyDeviceToHost, lat->st));
+  QF_CUDA(lat, cudaStreamSynchronize(lat->st));
+  if (err) {
+    QF_CUDA(lat, cudaMemsetAsync(&lat->sc()->err[0], 0, sizeof(int), lat->st));
+    return fail(lat, QF_ETIMEOUT, "a bounded device wait ran out (the blocks of a cluster lost each other)");
+  }
+  return QF_OK;
+}
+
 // ---- two FDTD steps per pass (complex FP32) ----------------------------------------------
 static void tb_args(qf_lattice* lat, const double* scale, StencilTbArgs& g) {
   const double a = lat->d.a, m = lat->mass, dt = lat->dtau;
@@ -641,6 +680,27 @@ static cudaError_t fdtd_pair(qf_lattice* lat, const double* scale) {
   return launch(lat, K_STENCIL_2STEP, [&] { return launch_stencil_tb(g, lat->st); });
 }
 
+// nsteps resident steps of the live psi in one launch (with sums: one step and its partial
+// rows); `scale` applies to the first.
+static cudaError_t res_steps(qf_lattice* lat, int nsteps, bool reduce, const double* scale, int* nblocks) {
+  ResGroup g;
+  g.count = 1;
+  g.a[0] = res_args(lat, scale, nsteps);
+  lat->xfwd_valid = false;
+  if (nblocks) *nblocks = fft_res_blocks(lat->d.n);
+  return launch(lat, K_FFT_RES, [&] { return launch_fft_res(lat->d.n, g, lat->v_real, reduce, lat->st); });
+}
+
+// How many steps of a resident lattice one launch takes from step t on: up to the next check,
+// the next snapshot or `left`, and no more than a launch of some milliseconds.  t is not a
+// check step.
+static int64_t res_run(int64_t t, int64_t left, int check_every, int snap_every) {
+  int64_t k = std::min<int64_t>(left, 2048);
+  if (check_every > 0) k = std::min<int64_t>(k, check_every - t % check_every);
+  if (snap_every > 0) k = std::min<int64_t>(k, snap_every - t % snap_every);
+  return k;
+}
+
 // One kinetic application on `in` (psi' written to `out` when write), with FP64 sums
 // when reduce; returns the number of partial rows written through nblocks.
 static cudaError_t kinetic_pass(qf_lattice* lat, void* in, void* out, bool write, bool reduce, const double* scale,
@@ -658,6 +718,7 @@ static cudaError_t kinetic_pass(qf_lattice* lat, void* in, void* out, bool write
     if (!stencil_group_member(lat, in, out, write, reduce, scale, g)) return cudaErrorInvalidValue;
     return launch(lat, kind, [&] { return launch_stencil<double>(g, lat->st); });
   }
+  if (uses_res(lat) && write && in == lat->psi()) return res_steps(lat, 1, reduce, scale, nblocks);
   // FFT terms: in place on `in` (out must equal in when writing); the scratch field is tmp.
   // A step on the live psi emits the next step's first pass and may skip its own.
   tune_fft_tiles(lat);  // first four-pass step of this size in the process (overwrites tmp)
@@ -774,6 +835,21 @@ static cudaError_t after_pair(qf_lattice* lat, int snap_every, cudaStream_t st) 
   lat->live = 1 - lat->live;
   lat->clean = true;
   for (int i = 0; i < 2; ++i) {
+    lat->step += 1;
+    lat->tau += lat->dtau;
+  }
+  return take_snapshot(lat, snap_every, st);
+}
+
+// Bookkeeping after k steps without a check in one launch (a snapshot at most after the last).
+static cudaError_t after_run(qf_lattice* lat, int64_t k, int snap_every, cudaStream_t st) {
+  if (lat->pending_scale) {
+    lat->K += lat->jcur - lat->K_check;
+    lat->renorm_step = lat->step;
+  }
+  lat->K += k * lat->kcur;
+  lat->pending_scale = false;
+  for (int64_t i = 0; i < k; ++i) {
     lat->step += 1;
     lat->tau += lat->dtau;
   }
@@ -916,6 +992,13 @@ extern "C" qf_status qf_step_n(qf_lattice* lat, int64_t max_steps, double tol_ab
       done += 2;
       continue;
     }
+    if (!check && uses_res(lat)) {
+      const int64_t k = res_run(t, max_steps - done, check_every, snap_every);
+      QF_CUDA(lat, res_steps(lat, (int)k, false, scale, nullptr));
+      QF_CUDA(lat, after_run(lat, k, snap_every, lat->st));
+      done += k;
+      continue;
+    }
     int nb = 0;
     void* in = lat->psi();
     void* out = fdtd ? lat->tmp() : in;
@@ -963,8 +1046,14 @@ extern "C" qf_status qf_step_n(qf_lattice* lat, int64_t max_steps, double tol_ab
     }
   }
   if (steps_done) *steps_done = done;
-  // surface asynchronous launch failures before reporting (no kernel of a step waits on another)
-  QF_CUDA(lat, cudaStreamSynchronize(lat->st));
+  // surface asynchronous launch failures and bounded-wait time-outs (resident steps only: no
+  // other kernel waits on another block) before reporting
+  if (uses_res(lat)) {
+    const qf_status s = check_device_error(lat);
+    if (s != QF_OK) return s;
+  } else {
+    QF_CUDA(lat, cudaStreamSynchronize(lat->st));
+  }
   return status;
 }
 
@@ -1323,7 +1412,7 @@ struct qf_batch {
     int64_t max_steps, steps_done;
     double tol_abs, tol_rel;
     int status;  // QF_BATCH_RUNNING, QF_OK (converged), QF_ENOTCONV (step cap reached)
-    bool mid_pair;  // advanced two steps by the previous batch step's launch: sits this one out
+    int ahead;   // steps already taken by an earlier batch step's launch: sits as many out
   };
   cudaStream_t st = nullptr;
   std::vector<Member> m;
@@ -1381,7 +1470,7 @@ extern "C" qf_status qf_batch_add(qf_batch* b, qf_lattice* lat, int64_t max_step
     if (x.lat == lat) return bfail(b, QF_EINVAL, "lattice already in the batch");
   // work of the lattice's own stream must be visible to the batch stream
   QF_BCUDA(b, cudaStreamSynchronize(lat->st));
-  b->m.push_back({lat, max_steps, 0, tol_abs, tol_rel, QF_BATCH_RUNNING, false});
+  b->m.push_back({lat, max_steps, 0, tol_abs, tol_rel, QF_BATCH_RUNNING, 0});
   b->drop_graphs();
   return QF_OK;
 }
@@ -1415,18 +1504,18 @@ static bool pairable(const qf_lattice* L) {
 }
 
 // Issues the launches of one batch step for the running members `run` (check flags chk);
-// nblk receives each member's partial rows.  pm (optional, per member of run) selects the
-// FDTD members' form: 0 one step, 1 two steps in one pass (psi_{t+2} into the scratch
-// field; the caller skips the member in the next batch step), 2 nothing (the second step
-// of a pair issued in the previous batch step).  Host state is touched only where later
-// launches depend on it (xfwd_valid of FFT members).
+// nblk receives each member's partial rows.  ns (per member of run) is the number of steps its
+// launch takes: 1; 2 for FDTD members (two steps in one pass, psi_{t+2} into the scratch
+// field) and any number for resident FFT members (the caller then skips the member in as
+// many batch steps less one); 0 for nothing (such a skipped step).  Host state is touched
+// only where later launches depend on it (xfwd_valid of FFT members).
 static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, const std::vector<char>& chk,
-                                  std::vector<int>& nblk, cudaStream_t st, const std::vector<char>* pm = nullptr) {
+                                  std::vector<int>& nblk, cudaStream_t st, const std::vector<int>& ns) {
   const int R = (int)run.size();
   // group FP32 members by (N, kinetic family, real V, check); FP64 members run alone
   std::vector<char> done(R, 0);
   for (int k = 0; k < R; ++k) {
-    if (done[k]) continue;
+    if (done[k] || ns[k] == 0) continue;
     qf_lattice* L = b->m[run[k]].lat;
     const double* sk = L->pending_scale ? &L->sc()->scale[1] : &L->sc()->scale[2];
     const bool fdtd = L->kinetic == QF_KIN_FDTD;
@@ -1440,12 +1529,13 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
     }
     std::vector<int> g;
     for (int q = k; q < R; ++q) {
-      if (done[q]) continue;
+      if (done[q] || ns[q] == 0) continue;
       qf_lattice* M = b->m[run[q]].lat;
       // complex-FP32 FDTD members of any size share a launch (the stencil kernel takes
       // each member's N from its block table); FFT members need the same plan (N)
       if (!M->c64() || (M->kinetic == QF_KIN_FDTD) != fdtd || (!fdtd && M->d.n != L->d.n)) continue;
-      if (!fdtd && (M->v_real != L->v_real || chk[q] != chk[k] || uses_fft2(M) != uses_fft2(L))) continue;
+      if (!fdtd && (M->v_real != L->v_real || chk[q] != chk[k] || uses_fft2(M) != uses_fft2(L) || uses_res(M) != uses_res(L)))
+        continue;
       g.push_back(q);
       done[q] = 1;
     }
@@ -1461,10 +1551,8 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
         for (int j = 0; j < cnt; ++j) {
           const int q = g[off + j];
           qf_lattice* M = b->m[run[q]].lat;
-          const int mode = pm ? (*pm)[q] : 0;
           const double* sq = M->pending_scale ? &M->sc()->scale[1] : &M->sc()->scale[2];
-          if (mode == 2) continue;
-          if (mode == 1) {
+          if (ns[q] == 2) {
             StencilTbGroup& t = tg[M->v_real ? 1 : 0];
             tb_args(M, sq, t.m[t.count++]);
             continue;
@@ -1482,6 +1570,18 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
             QF_BCUDA(b, launch_stencil_tb(t, st));
             b->launches += 1;
           }
+      } else if (uses_res(L)) {
+        ResGroup rg;
+        rg.count = cnt;
+        for (int j = 0; j < cnt; ++j) {
+          const int q = g[off + j];
+          qf_lattice* M = b->m[run[q]].lat;
+          rg.a[j] = res_args(M, M->pending_scale ? &M->sc()->scale[1] : &M->sc()->scale[2], ns[q]);
+          M->xfwd_valid = false;
+          nblk[q] = fft_res_blocks(n);
+        }
+        QF_BCUDA(b, launch_fft_res(n, rg, L->v_real, chk[k], st));
+        b->launches += 1;
       } else {
         const bool two = uses_fft2(L);
         tune_fft_tiles(L);  // (runs once per size; never inside a capture)
@@ -1541,7 +1641,7 @@ static qf_status batch_chunk_graph(qf_batch* b, const std::vector<int>& run, int
       return QF_OK;
     key.push_back(reinterpret_cast<uintptr_t>(L));
     key.push_back((uintptr_t)((L->live & 1) | (L->xfwd_valid ? 2 : 0) | (uses_fft2(L) ? 4 : 0) |
-                              (pairable(L) ? 8 : 0)));
+                              (pairable(L) ? 8 : 0) | (uses_res(L) ? 16 : 0)));
   }
   std::vector<char> pair(run.size(), 0);
   for (size_t q = 0; q < run.size(); ++q) {
@@ -1564,17 +1664,18 @@ static qf_status batch_chunk_graph(qf_batch* b, const std::vector<int>& run, int
       saved.push_back({L->live, L->clean, L->xfwd_valid, L->pending_scale, L->launches});
     }
     const int64_t l0 = b->launches;
-    std::vector<char> nochk(run.size(), 0), pm(run.size(), 0);
-    std::vector<int> nblk(run.size(), 0);
+    std::vector<char> nochk(run.size(), 0);
+    std::vector<int> nblk(run.size(), 0), ns(run.size(), 1);
     cudaGraph_t graph = nullptr;
     QF_BCUDA(b, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     qf_status s = QF_OK;
     for (int j = 0; j < k && s == QF_OK; ++j) {
-      for (size_t q = 0; q < run.size(); ++q) pm[q] = !pair[q] ? 0 : (j & 1) ? 2 : (j + 1 < k) ? 1 : 0;
-      s = batch_issue_step(b, run, nochk, nblk, st, &pm);
+      for (size_t q = 0; q < run.size(); ++q)
+        ns[q] = pair[q] ? ((j & 1) ? 0 : (j + 1 < k) ? 2 : 1) : uses_res(b->m[run[q]].lat) ? (j == 0 ? k : 0) : 1;
+      s = batch_issue_step(b, run, nochk, nblk, st, ns);
       for (size_t q = 0; q < run.size(); ++q) {
         qf_lattice* L = b->m[run[q]].lat;
-        if (pm[q] == 2) continue;
+        if (ns[q] == 0) continue;
         L->pending_scale = false;
         if (L->kinetic == QF_KIN_FDTD) L->live = 1 - L->live;
       }
@@ -1658,14 +1759,14 @@ extern "C" qf_status qf_batch_step(qf_batch* b, int64_t steps, int check_every, 
   std::vector<double> tau_t;
   std::vector<int64_t> t_of;
   std::vector<double> e3;
-  std::vector<char> pm;
+  std::vector<int> ns;
   for (int64_t s = 0; s < steps; ++s) {
     run.clear();
     bool any = false;
     for (int i = 0; i < (int)b->m.size(); ++i)
       if (b->m[i].status == QF_BATCH_RUNNING) {
-        if (b->m[i].mid_pair) {
-          b->m[i].mid_pair = false;  // this step was the second of its pair
+        if (b->m[i].ahead > 0) {
+          b->m[i].ahead -= 1;  // an earlier launch took this step
           any = true;
         } else if (b->m[i].steps_done >= b->m[i].max_steps) {
           b->m[i].status = QF_ENOTCONV;
@@ -1691,28 +1792,31 @@ extern "C" qf_status qf_batch_step(qf_batch* b, int64_t steps, int check_every, 
     nblk.assign(R, 0);
     tau_t.assign(R, 0);
     t_of.assign(R, 0);
-    pm.assign(R, 0);
+    ns.assign(R, 1);
     for (int k = 0; k < R; ++k) {
       const auto& mb = b->m[run[k]];
       qf_lattice* L = mb.lat;
       t_of[k] = L->step;
       tau_t[k] = L->tau;
       chk[k] = check_every > 0 && L->step % check_every == 0;
-      // two FDTD steps in one launch where a lone lattice would pair them too
+      // as many steps in one launch as a lone lattice would take
       if (s + 2 <= steps && mb.steps_done + 2 <= mb.max_steps && fuse_pair(L, L->step, check_every, snap_every))
-        pm[k] = 1;
+        ns[k] = 2;
+      else if (!chk[k] && uses_res(L))
+        ns[k] = (int)res_run(L->step, std::min(steps - s, mb.max_steps - mb.steps_done), check_every, snap_every);
     }
-    qf_status is = batch_issue_step(b, run, chk, nblk, st, &pm);
+    qf_status is = batch_issue_step(b, run, chk, nblk, st, ns);
     if (is != QF_OK) return is;
     // per-member bookkeeping, identical to qf_step_n
     bool any_check = false;
     for (int k = 0; k < R; ++k) {
       auto& mb = b->m[run[k]];
       qf_lattice* L = mb.lat;
-      if (pm[k]) {
-        QF_BCUDA(b, after_pair(L, snap_every, st));
-        mb.steps_done += 2;
-        mb.mid_pair = true;
+      if (ns[k] > 1 || (!chk[k] && uses_res(L))) {
+        if (L->kinetic == QF_KIN_FDTD) QF_BCUDA(b, after_pair(L, snap_every, st));
+        else QF_BCUDA(b, after_run(L, ns[k], snap_every, st));
+        mb.steps_done += ns[k];
+        mb.ahead = ns[k] - 1;
         continue;
       }
       QF_BCUDA(b, after_step(L, chk[k], nblk[k], snap_every, st));
@@ -1735,6 +1839,11 @@ extern "C" qf_status qf_batch_step(qf_batch* b, int64_t steps, int check_every, 
     }
   }
   QF_BCUDA(b, cudaStreamSynchronize(st));
+  for (auto& x : b->m)
+    if (uses_res(x.lat)) {
+      const qf_status es = check_device_error(x.lat);
+      if (es != QF_OK) return bfail(b, es, x.lat->err);
+    }
   int nr = 0;
   for (auto& x : b->m) {
     if (x.status == QF_BATCH_RUNNING && x.steps_done >= x.max_steps) x.status = QF_ENOTCONV;

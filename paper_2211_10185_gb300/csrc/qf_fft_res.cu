@@ -1,0 +1,105 @@
+// Launchers of the resident FFT steps (kernels in qf_fft_res.cuh).
+#include "qf_fft_res.cuh"
+
+namespace qf {
+
+template <int N, typename K>
+static cudaError_t res_launch(K kern, int members, cudaStream_t st, const void* arg) {
+  using G = ResG<N>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(G::C, members);
+  cfg.blockDim = dim3(G::THREADS);
+  cfg.dynamicSmemBytes = G::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = G::C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  void* args[] = {const_cast<void*>(arg)};
+  return cudaLaunchKernelExC(&cfg, (const void*)kern, args);
+}
+
+// Shared-memory and cluster limits of every variant of size N; whether the device can hold a
+// cluster at all (16 blocks exceed the portable 8).
+template <int N>
+static bool res_setup() {
+  using G = ResG<N>;
+  const void* k[] = {(const void*)fft_res_kernel<N, true, true>, (const void*)fft_res_kernel<N, true, false>,
+                     (const void*)fft_res_kernel<N, false, true>, (const void*)fft_res_kernel<N, false, false>,
+                     (const void*)fft_res_static_kernel<N, true, true>, (const void*)fft_res_static_kernel<N, true, false>,
+                     (const void*)fft_res_static_kernel<N, false, true>, (const void*)fft_res_static_kernel<N, false, false>};
+  bool ok = true;
+  for (const void* f : k) {
+    ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G::C);
+    cfg.blockDim = dim3(G::THREADS);
+    cfg.dynamicSmemBytes = G::SMEM;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = G::C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    ok = ok && cudaOccupancyMaxActiveClusters(&clusters, f, &cfg) == cudaSuccess && clusters > 0;
+  }
+  cudaGetLastError();  // (a refusal above is an answer, not an error)
+  return ok;
+}
+template <int N>
+static bool res_ready() {
+  static const bool ok = res_setup<N>();
+  return ok;
+}
+
+#define QF_RES_CASES QF_CASE(8) QF_CASE(12) QF_CASE(16) QF_CASE(24) QF_CASE(32)
+
+int fft_res_blocks(int n) {
+  switch (n) {
+#define QF_CASE(NN) \
+  case NN:          \
+    return res_ready<NN>() ? ResG<NN>::C : 0;
+    QF_RES_CASES
+#undef QF_CASE
+    default:
+      return 0;
+  }
+}
+
+cudaError_t launch_fft_res(int n, const ResGroup& g, bool v_real, bool reduce, cudaStream_t st) {
+  if (g.count < 1 || g.count > kGroupMax || fft_res_blocks(n) == 0) return cudaErrorInvalidValue;
+  switch (n) {
+#define QF_CASE(NN)                                                                                          \
+  case NN:                                                                                                   \
+    return res_launch<NN>(v_real ? (reduce ? fft_res_kernel<NN, true, true> : fft_res_kernel<NN, true, false>) \
+                                 : (reduce ? fft_res_kernel<NN, false, true> : fft_res_kernel<NN, false, false>), \
+                          g.count, st, &g);
+    QF_RES_CASES
+#undef QF_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_fft_res_static(int n, const ResStatic& g, bool v_real, bool reduce, cudaStream_t st) {
+  if (fft_res_blocks(n) == 0) return cudaErrorInvalidValue;
+  switch (n) {
+#define QF_CASE(NN)                                                                                                  \
+  case NN:                                                                                                           \
+    return res_launch<NN>(v_real ? (reduce ? fft_res_static_kernel<NN, true, true> : fft_res_static_kernel<NN, true, false>) \
+                                 : (reduce ? fft_res_static_kernel<NN, false, true> : fft_res_static_kernel<NN, false, false>), \
+                          1, st, &g);
+    QF_RES_CASES
+#undef QF_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace qf

@@ -1,0 +1,374 @@
+// Resident imaginary-time FFT steps for small complex-FP32 lattices (N <= 32; Eqs. HK1-HK3
+// and the update of Sec. 2), sm_103a.
+//
+// One thread-block cluster holds a whole lattice and takes any number of steps per launch:
+// psi and V stay in registers, the transformed field in shared memory, and the two
+// redistributions of a step go through distributed shared memory.  Each of the cluster's C
+// blocks owns P = N / C z-planes; a thread transforms whole lines in registers:
+//   x forward, y forward on its planes  ->  column (kx, ky) to the block that owns ky
+//   z forward, T(k), z inverse          ->  column element z to the block that owns z
+//   y inverse, x inverse, update of psi in registers, and round again.
+// A step has two block barriers and no cluster barrier: an element is stored into the block
+// that needs it (st.async), whose barrier counts the bytes, and a block goes on when all of
+// its P N^2 elements are in.  Nothing is overwritten early: a block stores into the buffer
+// that a peer read last only after it has received everything that the peer sends once it
+// has read it.
+//
+// What bounds it: instruction issue and latency of few warps (N = 32: two per SM on 16 SMs).
+// The four-pass form needs four launches a step, each bound by the 2-3 us that any kernel
+// takes.  One step, before and now: N = 8: 7.0 / 1.6 us, 12: 11.2 / 2.1, 16: 13.0 / 2.2, 24:
+// 14.8 / 4.2, 32: 11.6 / 5.3.  At N = 48 (13.3 against 12.8 us) the 16 SMs of a cluster are too few.
+#pragma once
+#include <utility>
+
+#include "qf_fft_impl.cuh"
+
+namespace qf {
+
+// Lattices per launch and their arguments.  Members run on clusters of their own and need
+// not be stepped alike (nsteps, reduce).
+struct ResArgs {
+  cpx<float>* psi;           // psi_t in, psi_{t + nsteps} out
+  const void* v;             // potential: cpx<float> or float
+  const float* symbol;       // per-axis kinetic symbol
+  const double* scale;       // output scale of the first step
+  const double* scale2;      // and of the others
+  double* partials;          // kNumSums per block of the cluster when reducing
+  float tcoef, am2, half_dtau, dtau;
+  int* err;                  // set to 1 when a bounded wait ran out
+  int kinetic, nsteps;
+};
+struct ResGroup {
+  int count;
+  ResArgs a[kGroupMax];
+};
+// One step of a caller that keeps no tables: they travel in the kernel's parameters.
+struct ResStatic {
+  ResArgs a;
+  float sym[32];
+  double out_scale;
+};
+
+constexpr bool res_supported(int n) { return n == 8 || n == 12 || n == 16 || n == 24 || n == 32; }
+
+template <int N>
+struct ResG {
+  static constexpr int C = N == 8 ? 2 : N == 12 ? 4 : N <= 24 ? 8 : 16;  // blocks per cluster
+  static constexpr int P = N / C;
+  static constexpr int THREADS = P * N;  // one line each
+  // row pitch in elements: odd, so that lanes along a column and along a row both spread
+  // over all banks
+  static constexpr int NP = N + 1;
+  static constexpr int SLAB = N * NP;  // a plane [y][x], or a ky [z][kx]
+  static constexpr unsigned BYTES = P * N * N * 8;  // a block's share of a redistribution
+  static constexpr size_t SMEM = (size_t)2 * P * SLAB * 8 + N * 8 + 32 * kNumSums * 8;
+  static_assert(N % C == 0 && THREADS <= 1024, "resident geometry");
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// Stores into the shared memory of block `rank` of the cluster, at the place `p` has in this
+// one's, and counts the bytes on that block's barrier at the place of `bar`.
+__device__ __forceinline__ unsigned res_map(const void* p, int rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(cpx<float>* p, int rank, cpx<float> v, const unsigned long long* bar) {
+  unsigned long long w;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "f"(v.x), "f"(v.y));
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];\n" ::"r"(res_map(p, rank)),
+               "l"(w), "r"(res_map(bar, rank))
+               : "memory");
+}
+// Bounded wait for phase `parity` of the block's own barrier (acquires what the cluster's
+// blocks stored); after a time-out it returns false at once for the rest of the launch.
+__device__ __forceinline__ bool res_wait(unsigned long long* bar, unsigned parity, bool ok) {
+  const unsigned b = (unsigned)__cvta_generic_to_shared(bar);
+  for (unsigned it = 0; ok && it < (1u << 24); ++it) {
+    unsigned done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done)
+                 : "r"(b), "r"(parity)
+                 : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void res_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(bytes)
+               : "memory");
+}
+
+// ---- transforms of N points in a thread's registers ----------------------------------------
+// Packed complex FP32 sums: one instruction for both parts.
+__device__ __forceinline__ cpx<float> rc_add(cpx<float> a, cpx<float> b) {
+  cpx<float> r;
+  asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ cpx<float> rc_sub(cpx<float> a, cpx<float> b) {
+  cpx<float> r;
+  asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+// cos and sin of 2 pi k / n, 0 <= k < n, from their Taylor series on [0, pi/4]
+constexpr double rc_series(double x, bool sine) {
+  double t = sine ? x : 1.0, s = t;
+  for (int i = sine ? 3 : 2; i < 24; i += 2) {
+    t *= -x * x / (double)(i * (i - 1));
+    s += t;
+  }
+  return s;
+}
+constexpr double rc_cos(int k, int n) {
+  const int o = 8 * k / n;                                  // octant
+  const double x = 6.283185307179586476925286766559 / n;
+  switch (o) {
+    case 0: return rc_series(x * k, false);
+    case 1: return rc_series(x * (n / 4.0 - k), true);
+    case 2: return -rc_series(x * (k - n / 4.0), true);
+    case 3: return -rc_series(x * (n / 2.0 - k), false);
+    case 4: return -rc_series(x * (k - n / 2.0), false);
+    case 5: return -rc_series(x * (3.0 * n / 4.0 - k), true);
+    case 6: return rc_series(x * (k - 3.0 * n / 4.0), true);
+    default: return rc_series(x * (n - k), false);
+  }
+}
+constexpr double rc_sin(int k, int n) { return rc_cos((k + n - n / 4) % n, n); }  // (n a multiple of 4)
+
+template <bool INV>
+__device__ __forceinline__ void rc_dft4(cpx<float>& x0, cpx<float>& x1, cpx<float>& x2, cpx<float>& x3) {
+  const cpx<float> a0 = rc_add(x0, x2), a1 = rc_sub(x0, x2), a2 = rc_add(x1, x3), d = rc_sub(x1, x3);
+  x0 = rc_add(a0, a2);
+  x2 = rc_sub(a0, a2);
+  const cpx<float> p = mk<float>(a1.x + d.y, a1.y - d.x), q = mk<float>(a1.x - d.y, a1.y + d.x);  // a1 -+ i d
+  x1 = INV ? q : p;
+  x3 = INV ? p : q;
+}
+template <bool INV>
+__device__ __forceinline__ void rc_dft3(cpx<float>& x0, cpx<float>& x1, cpx<float>& x2) {
+  const float h = 0.86602540378443864676f;  // sin(2 pi / 3)
+  const cpx<float> s = rc_add(x1, x2), d = rc_sub(x1, x2);
+  const cpx<float> t = mk<float>(fmaf(-0.5f, s.x, x0.x), fmaf(-0.5f, s.y, x0.y));
+  x0 = rc_add(x0, s);
+  const cpx<float> p = mk<float>(fmaf(h, d.y, t.x), fmaf(-h, d.x, t.y)), q = mk<float>(fmaf(-h, d.y, t.x), fmaf(h, d.x, t.y));
+  x1 = INV ? q : p;
+  x2 = INV ? p : q;
+}
+// a exp(-+ 2 pi i K / N)
+template <int K, int N, bool INV>
+__device__ __forceinline__ cpx<float> rc_rot(cpx<float> a) {
+  constexpr int k = K % N;
+  if constexpr (k == 0) return a;
+  else if constexpr (4 * k == N) return INV ? mk<float>(-a.y, a.x) : mk<float>(a.y, -a.x);
+  else if constexpr (2 * k == N) return mk<float>(-a.x, -a.y);
+  else if constexpr (4 * k == 3 * N) return INV ? mk<float>(a.y, -a.x) : mk<float>(-a.y, a.x);
+  else return rot<float, INV>(a, (float)rc_cos(k, N), (float)rc_sin(k, N));
+}
+template <int N, bool INV, int STRIDE>
+__device__ __forceinline__ void rc_dft(cpx<float>* x);
+// N = A B by decimation: A-point transforms over n1 of n = B n1 + n2, twiddles, B-point ones
+// over n2, output k = k1 + A k2.  x[STRIDE i] holds element i before and after.
+template <int N, int A, int B, bool INV, int STRIDE, int... I2, int... I1>
+__device__ __forceinline__ void rc_split(cpx<float>* x, std::integer_sequence<int, I2...>, std::integer_sequence<int, I1...>) {
+  (rc_dft<A, INV, STRIDE * B>(x + STRIDE * I2), ...);
+  auto twiddle = [&](auto n2c) {
+    constexpr int n2 = decltype(n2c)::value;
+    ((x[STRIDE * (B * I1 + n2)] = rc_rot<n2 * I1, N, INV>(x[STRIDE * (B * I1 + n2)])), ...);
+  };
+  (twiddle(std::integral_constant<int, I2>{}), ...);
+  (rc_dft<B, INV, STRIDE>(x + STRIDE * B * I1), ...);
+  cpx<float> y[N];
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1)
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) y[k1 + A * k2] = x[STRIDE * (B * k1 + k2)];
+#pragma unroll
+  for (int k = 0; k < N; ++k) x[STRIDE * k] = y[k];
+}
+template <int N, bool INV, int STRIDE>
+__device__ __forceinline__ void rc_dft(cpx<float>* x) {
+  if constexpr (N == 2) {
+    const cpx<float> d = rc_sub(x[0], x[STRIDE]);
+    x[0] = rc_add(x[0], x[STRIDE]);
+    x[STRIDE] = d;
+  } else if constexpr (N == 3) {
+    rc_dft3<INV>(x[0], x[STRIDE], x[2 * STRIDE]);
+  } else if constexpr (N == 4) {
+    rc_dft4<INV>(x[0], x[STRIDE], x[2 * STRIDE], x[3 * STRIDE]);
+  } else {
+    constexpr int A = N == 8 ? 4 : N == 16 ? 4 : N == 32 ? 4 : 3, B = N / A;  // 12, 24: 3 x
+    rc_split<N, A, B, INV, STRIDE>(x, std::make_integer_sequence<int, B>{}, std::make_integer_sequence<int, A>{});
+  }
+}
+
+// The block's sums (THREADS need not fill its last warp) to out[0 .. kNumSums).
+template <int THREADS>
+__device__ __forceinline__ void res_block_sum(double (&s)[kNumSums], double* scratch, double* out) {
+  constexpr int WARPS = (THREADS + 31) / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lanes = warp + 1 < WARPS ? 32 : THREADS - 32 * (WARPS - 1);
+  const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int i = 0; i < kNumSums; ++i) {
+      const double t = __shfl_down_sync(mask, s[i], off);
+      if (lane + off < lanes) s[i] += t;
+    }
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < kNumSums; ++i) scratch[warp * kNumSums + i] = s[i];
+  __syncthreads();
+  if (threadIdx.x < kNumSums) {
+    double t = 0.0;
+    for (int w = 0; w < WARPS; ++w) t += scratch[w * kNumSums + threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+}
+
+template <int N, bool VREAL, bool SUMS>
+__device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, float sc1, float sc2) {
+  using G = ResG<N>;
+  constexpr int P = G::P, NP = G::NP;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* red_s = reinterpret_cast<double*>(smem_raw);
+  cpx<float>* plane = reinterpret_cast<cpx<float>*>(red_s + 32 * kNumSums);  // [z_l][y][x]
+  cpx<float>* cols = plane + P * G::SLAB;                                    // [ky_l][z][kx]
+  float* sym = reinterpret_cast<float*>(cols + P * G::SLAB);
+  __shared__ alignas(8) unsigned long long bars[2];  // data in cols, in plane
+  const int tid = threadIdx.x, rank = blockIdx.x;
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&bars[i])) : "memory");
+      res_expect(&bars[i], G::BYTES);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  bool ok = true;
+  unsigned parity = 0;
+  for (int i = tid; i < N; i += G::THREADS) sym[i] = sym_g[i];
+  // the thread's line: row `l` of slab `s` as an x line, column `l` of slab s as a y or z line
+  const int s = tid / N, l = tid % N;
+  cpx<float>* xline = plane + s * G::SLAB + l * NP;
+  cpx<float>* ycol = plane + s * G::SLAB + l;
+  cpx<float>* zcol = cols + s * G::SLAB + l;
+  const long long row = (((long long)rank * P + s) * N + l) * N;
+  // psi and V of the line
+  cpx<float> v[N], psi[N];
+  float vr[N], vi[VREAL ? 1 : N];
+#pragma unroll
+  for (int x = 0; x < N; ++x) {
+    psi[x] = a.psi[row + x];
+    if constexpr (VREAL) {
+      vr[x] = reinterpret_cast<const float*>(a.v)[row + x];
+    } else {
+      const cpx<float> w = reinterpret_cast<const cpx<float>*>(a.v)[row + x];
+      vr[x] = w.x;
+      vi[x] = w.y;
+    }
+  }
+  cluster_sync();  // the symbol is in place, and every block of the cluster is running
+  for (int t = 0; t < (SUMS ? 1 : a.nsteps); ++t) {
+    // One copy of the transform's code a direction for the longer lines: with 2-3 warps per SM
+    // straight code of all six ran at the pace of the instruction cache (N = 32: 6.4 us a step,
+    // 5.3 so; N = 24: 4.4 and 4.2; N = 16: 2.2 straight, 2.4 so).
+    constexpr int kUnroll = N <= 16 ? 3 : 1;
+#pragma unroll
+    for (int x = 0; x < N; ++x) v[x] = psi[x];
+#pragma unroll kUnroll
+    for (int ph = 0; ph < 3; ++ph) {  // x, y, z forward
+      rc_dft<N, false, 1>(v);
+      if (ph == 0) {
+#pragma unroll
+        for (int x = 0; x < N; ++x) xline[x] = v[x];
+        __syncthreads();
+#pragma unroll
+        for (int y = 0; y < N; ++y) v[y] = ycol[y * NP];
+      } else if (ph == 1) {
+#pragma unroll
+        for (int ky = 0; ky < N; ++ky)
+          st_cluster(cols + (ky % P) * G::SLAB + (rank * P + s) * NP + l, ky / P, v[ky], &bars[0]);
+        ok = res_wait(&bars[0], parity, ok);
+        if (tid == 0) res_expect(&bars[0], G::BYTES);
+#pragma unroll
+        for (int z = 0; z < N; ++z) v[z] = zcol[z * NP];
+      }
+    }
+    const float sxy = sym[l] + sym[rank * P + s];
+#pragma unroll
+    for (int z = 0; z < N; ++z) v[z] = cscale<float>(v[z], kin_mult<float>(a.kinetic, sxy, sym[z], a.tcoef, a.am2));
+#pragma unroll kUnroll
+    for (int ph = 0; ph < 3; ++ph) {  // z, y, x inverse
+      rc_dft<N, true, 1>(v);
+      if (ph == 0) {
+#pragma unroll
+        for (int z = 0; z < N; ++z)
+          st_cluster(plane + (z % P) * G::SLAB + (rank * P + s) * NP + l, z / P, v[z], &bars[1]);
+        ok = res_wait(&bars[1], parity, ok);
+        if (tid == 0) res_expect(&bars[1], G::BYTES);
+        parity ^= 1;
+#pragma unroll
+        for (int y = 0; y < N; ++y) v[y] = ycol[y * NP];
+      } else if (ph == 1) {
+#pragma unroll
+        for (int y = 0; y < N; ++y) ycol[y * NP] = v[y];
+        __syncthreads();
+#pragma unroll
+        for (int x = 0; x < N; ++x) v[x] = xline[x];
+      }
+    }
+    // v = H_K psi at the sites of psi; update
+    if constexpr (SUMS) {
+      CheckSums<float> sum;
+#pragma unroll
+      for (int x = 0; x < N; ++x) sum.add(psi[x], v[x], mk<float>(vr[x], VREAL ? 0.f : vi[VREAL ? 0 : x]));
+      double acc[kNumSums];
+      sum.to(acc);
+      res_block_sum<G::THREADS>(acc, red_s, a.partials + (long long)rank * kPartialStride);
+    }
+    const float sc = t == 0 ? sc1 : sc2;
+#pragma unroll
+    for (int x = 0; x < N; ++x) {
+      // d = 1 + dtau V/2; coef_B = 1/d; coef_A = (2 - d)/d
+      if constexpr (VREAL) {
+        const float d = 1.f + a.half_dtau * vr[x];
+        const cpx<float> num = cscale<float>(psi[x], 2.f - d) - cscale<float>(v[x], a.dtau);
+        psi[x] = cscale<float>(num, __fdividef(sc, d));
+      } else {
+        const cpx<float> d = mk<float>(1.f + a.half_dtau * vr[x], a.half_dtau * vi[x]);
+        const cpx<float> num = cmul<float>(mk<float>(2.f - d.x, -d.y), psi[x]) - cscale<float>(v[x], a.dtau);
+        psi[x] = cscale<float>(cmulc<float>(num, d), __fdividef(sc, d.x * d.x + d.y * d.y));
+      }
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < N; ++x) a.psi[row + x] = psi[x];
+  if (!ok && a.err) atomicExch(a.err, 1);
+}
+
+template <int N, bool VREAL, bool SUMS>
+__global__ void __launch_bounds__(ResG<N>::THREADS) fft_res_kernel(const __grid_constant__ ResGroup g) {
+  const ResArgs& a = g.a[blockIdx.y];
+  res_body<N, VREAL, SUMS>(a, a.symbol, (float)*a.scale, (float)*a.scale2);
+}
+template <int N, bool VREAL, bool SUMS>
+__global__ void __launch_bounds__(ResG<N>::THREADS) fft_res_static_kernel(const __grid_constant__ ResStatic g) {
+  res_body<N, VREAL, SUMS>(g.a, g.sym, (float)g.out_scale, (float)g.out_scale);
+}
+
+// nsteps steps of every member of g (one lattice size, one kind of potential) in one launch;
+// with `reduce` one step and its check sums.
+cudaError_t launch_fft_res(int n, const ResGroup& g, bool v_real, bool reduce, cudaStream_t st);
+cudaError_t launch_fft_res_static(int n, const ResStatic& g, bool v_real, bool reduce, cudaStream_t st);
+// Partial-sum rows of a member; 0 where the size has no resident form or the device cannot
+// run its cluster.
+int fft_res_blocks(int n);
+
+}  // namespace qf

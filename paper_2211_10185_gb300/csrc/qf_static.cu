@@ -23,6 +23,7 @@
 
 #include "../../include/qfdtd.h"
 #include "qf_common.cuh"
+#include "qf_fft_res.cuh"
 
 namespace qf {
 namespace {
@@ -85,6 +86,30 @@ __global__ void static_tables_kernel(const __grid_constant__ StaticTables t, flo
   }
 }
 
+// Both per-axis symbols of the sizes that run in one launch, computed once per process (they
+// depend on n alone).
+struct HostTables {
+  float naive[32] = {}, sine[32] = {};
+  explicit HostTables(int n) {
+    for (int j = 0; j < n; ++j) {
+      const double k = 2.0 * M_PI * (double)(j <= n / 2 ? j : j - n) / (double)n;
+      naive[j] = (float)(k * k);
+      sine[j] = (float)(4.0 * sin(0.5 * k) * sin(0.5 * k));
+    }
+  }
+};
+const HostTables& host_tables(int n) {
+  static const HostTables t8(8), t12(12), t16(16), t24(24), t32(32);
+  return n == 8 ? t8 : n == 12 ? t12 : n == 16 ? t16 : n == 24 ? t24 : t32;
+}
+
+qf_status static_sums(const double* partials, int nb, DevScalars* dsc, double* sums, cudaStream_t st) {
+  if (launch_finish(partials, nb, dsc, 0, st) != cudaSuccess) return QF_ECUDA;
+  if (cudaMemcpyAsync(sums, dsc->sums, kNumSums * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+    return QF_ECUDA;
+  return QF_OK;
+}
+
 }  // namespace
 }  // namespace qf
 
@@ -100,6 +125,30 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
   void* base_v = nullptr;
   if (scratch_address(&base_v) != cudaSuccess) return QF_ECUDA;
   char* base = static_cast<char*>(base_v);
+
+  const double n3 = (double)n * n * n;
+  const float tcoef = (float)(kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3));
+  const float am2 = (float)((a * mass) * (a * mass));
+  DevScalars* dsc = reinterpret_cast<DevScalars*>(base + kStaticScOff);
+  double* partials = reinterpret_cast<double*>(base + kStaticPartialsOff);
+  if (const int nbr = fft_res_blocks(n); nbr > 0) {
+    // the whole step in one launch, its tables in the kernel's parameters
+    ResStatic r{};
+    const HostTables& t = host_tables(n);
+    memcpy(r.sym, kinetic == QF_KIN_FFT_NAIVE ? t.naive : t.sine, sizeof(r.sym));
+    r.out_scale = out_scale;
+    r.a.psi = static_cast<cpx<float>*>(psi);
+    r.a.v = v;
+    r.a.partials = partials;
+    r.a.tcoef = tcoef;
+    r.a.am2 = am2;
+    r.a.half_dtau = (float)(0.5 * dtau);
+    r.a.dtau = (float)dtau;
+    r.a.kinetic = kinetic;
+    r.a.nsteps = 1;
+    if (launch_fft_res_static(n, r, !v_complex, sums != nullptr, st) != cudaSuccess) return QF_ECUDA;
+    return sums ? static_sums(partials, nbr, dsc, sums, st) : QF_OK;
+  }
 
   // tables of this call (the array holds the previous call's): per-stage twiddles, the
   // per-axis symbol and the output scale, written on the device by the first launch
@@ -123,15 +172,12 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
   if (cudaLaunchKernel((const void*)static_tables_kernel, dim3(1), dim3(128), targs, 0, st) != cudaSuccess)
     return QF_ECUDA;
 
-  DevScalars* dsc = reinterpret_cast<DevScalars*>(base + kStaticScOff);
-  double* partials = reinterpret_cast<double*>(base + kStaticPartialsOff);
-  const double n3 = (double)n * n * n;
   FftPassArgs<float> p{};
   p.twiddle = reinterpret_cast<const cpx<float>*>(base + kStaticTwOff);
   p.symbol = reinterpret_cast<const float*>(base + kStaticSymOff);
   p.kinetic = kinetic;
-  p.tcoef = (float)(kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3));
-  p.am2 = (float)((a * mass) * (a * mass));
+  p.tcoef = tcoef;
+  p.am2 = am2;
   p.psi = static_cast<cpx<float>*>(psi);
   p.v = v;
   p.v_real = v_complex ? 0 : 1;
@@ -146,10 +192,5 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
   for (int pass = 0; pass < kFftPasses; ++pass)
     // (its twiddle scratch holds the first radix plan's table only)
     if (launch_fft_pass<float>(n, pass, p, tmp, st, &nb, false) != cudaSuccess) return QF_ECUDA;
-  if (sums) {
-    if (launch_finish(partials, nb, dsc, 0, st) != cudaSuccess) return QF_ECUDA;
-    if (cudaMemcpyAsync(sums, dsc->sums, kNumSums * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return QF_ECUDA;
-  }
-  return QF_OK;
+  return sums ? static_sums(partials, nb, dsc, sums, st) : QF_OK;
 }

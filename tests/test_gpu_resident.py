@@ -1,0 +1,108 @@
+"""Resident FFT steps (small complex-FP32 lattices, many steps per launch): every size, kinetic
+term and kind of potential against the four-pass form and the FP64 oracle, launches of
+different lengths against one, and the allocation-free step.
+
+Tolerances: a step's transforms carry about log2(N) roundings each way on top of the update's,
+so a step stays within 2e-6 (1 + log2 N) of FP64 in the 2-norm and s steps within s times
+that (the tolerance of the other FFT tests).  How the steps are cut into launches changes no
+operation: bitwise.
+"""
+import ctypes as C
+import math
+
+import numpy as np
+import pytest
+
+from oracle import qfdtd_oracle as O
+from paper_2211_10185_gb300 import inputs as I
+from paper_2211_10185_gb300 import qfdtd as Q
+
+pytestmark = pytest.mark.gpu
+SIZES = [8, 12, 16, 24, 32]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2211_10185_gb300 import build
+
+    build.build()
+
+
+def _inputs(n, complex_v):
+    a = 6.0 / n
+    v = I.cornell(n, a, 0.45, 0.2)
+    if complex_v:
+        v = v - 0.07j * np.abs(v)
+    return a, v, I.gaussian_field(n, n)
+
+
+def _gpu(n, a, v, psi0, kind, resident=True):
+    from paper_2211_10185_gb300.lattice import Lattice
+
+    lat = Lattice(n, a, precision="c64")
+    lat.set_potential(v)
+    lat.set_kinetic(kind, 0.9)
+    lat.set_wavefunction(psi0)
+    lat.use_two_pass_fft(resident)  # (off: the four-pass form)
+    return lat
+
+
+def _rel(a, b):
+    return np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel())
+
+
+@pytest.mark.parametrize("complex_v", [False, True])
+@pytest.mark.parametrize("kind", [O.FFT_NAIVE, O.FFT_SYMANZIK, O.FFT_REL])
+@pytest.mark.parametrize("n", SIZES)
+def test_resident_steps_match_four_pass_and_oracle(n, kind, complex_v):
+    a, v, psi0 = _inputs(n, complex_v)
+    steps, tol = 7, 2e-6 * (1 + math.log2(n)) * 7
+    ref = O.Lattice(n, a)
+    ref.set_potential(v.real, v.imag if complex_v else None)
+    ref.set_kinetic(kind, 0.9)
+    ref.set_wavefunction(psi0)
+    ref.step_n(steps, check_every=4, snap_every=0)
+    got = {}
+    for resident in (True, False):
+        lat = _gpu(n, a, v, psi0, kind, resident)
+        lat.step_n(steps, tol=0.0, check_every=4, snap_every=0)
+        got[resident] = lat.get_wavefunction()
+        assert _rel(got[resident], ref.psi) < tol
+        assert abs(lat.energies()["e"] - ref.energies()["e"]) < 1e-5 * abs(ref.energies()["e"])
+    assert _rel(got[True], got[False]) < 2 * tol
+
+
+@pytest.mark.parametrize("n", SIZES)
+def test_cutting_steps_into_launches_changes_no_bit(n):
+    a, v, psi0 = _inputs(n, False)
+    one, many = _gpu(n, a, v, psi0, O.FFT_SYMANZIK), _gpu(n, a, v, psi0, O.FFT_SYMANZIK)
+    one.step_n(40, tol=0.0, check_every=16, snap_every=0)
+    for k in (1, 2, 13, 1, 23):
+        many.step_n(k, tol=0.0, check_every=16, snap_every=0)
+    assert np.array_equal(one.get_wavefunction(), many.get_wavefunction())
+    assert one.energies() == many.energies()
+
+
+@pytest.mark.parametrize("complex_v", [False, True])
+@pytest.mark.parametrize("n", SIZES)
+def test_allocation_free_step_matches_resident_step(n, complex_v):
+    import torch
+
+    a, v, psi0 = _inputs(n, complex_v)
+    lat = _gpu(n, a, v, psi0, O.FFT_REL)
+    dt = lat.info()["dtau"]
+    lat.step_n(1, tol=0.0, check_every=0, snap_every=0)
+    psi = torch.from_numpy(psi0).to(torch.complex64).cuda()
+    vd = torch.from_numpy(v).to(torch.complex64 if complex_v else torch.float32).cuda()
+    sums = torch.empty(5, dtype=torch.float64, device="cuda")
+    st = Q.load().qf_fft_step_static(n, a, O.FFT_REL, 0.9, dt, C.c_void_p(psi.data_ptr()), C.c_void_p(vd.data_ptr()),
+                                     int(complex_v), 1.0, C.c_void_p(sums.data_ptr()), None)
+    assert st == Q.QF_OK
+    torch.cuda.synchronize()
+    # (one step of the same arithmetic in another instantiation, and the sums of its input)
+    assert _rel(psi.cpu().numpy().astype(np.complex128), lat.get_wavefunction()) < 2e-6 * (1 + math.log2(n))
+    assert abs(sums[0].item() - np.linalg.norm(psi0) ** 2) < 1e-6 * np.linalg.norm(psi0) ** 2
