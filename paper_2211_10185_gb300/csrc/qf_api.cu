@@ -25,6 +25,7 @@ namespace qf {
 bool fft2_supported(int n);
 int fft2_final_blocks(int n);
 int fft2_measure_blocks(int n);
+bool plane_supported(int n);
 cudaError_t launch_fft2_group_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
 cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st);
 cudaError_t launch_bounded_wait_probe(int* err, cudaStream_t st);
@@ -512,6 +513,13 @@ extern "C" qf_status qf_field_pointer(qf_lattice* lat, int slot, void** dev_ptr)
   return QF_OK;
 }
 
+// dtau of the update in the resident and plane forms (kinetic_dtau).
+static void form_dtau(const qf_lattice* lat, float tcoef, float* hi, float* lo) {
+  const double n3 = (double)lat->d.n * lat->d.n * lat->d.n, a = lat->d.a;
+  const double exact = lat->kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * lat->mass * n3);
+  kinetic_dtau(lat->d.n, lat->dtau, exact, tcoef, hi, lo);
+}
+
 // Arguments of the FFT passes / the stencil for one lattice (kernels in qf_fft_impl.cuh and
 // qf_stencil.cu); `in` is the field the kinetic term acts on.
 template <typename R>
@@ -535,6 +543,8 @@ static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduc
   p.write_psi = write ? 1 : 0;
   p.reduce = reduce ? 1 : 0;
   p.data = reinterpret_cast<cpx<R>*>(lat->tmp());
+  if constexpr (sizeof(R) == 4)
+    if (uses_fft2(lat) && plane_supported(lat->d.n)) form_dtau(lat, p.tcoef, &p.dtau, &p.dtau_lo);
   return p;
 }
 
@@ -551,7 +561,7 @@ static ResArgs res_args(qf_lattice* lat, const double* scale, int nsteps) {
   r.tcoef = p.tcoef;
   r.am2 = p.am2;
   r.half_dtau = p.half_dtau;
-  r.dtau = p.dtau;
+  form_dtau(lat, p.tcoef, &r.dtau, &r.dtau_lo);
   r.err = &lat->sc()->err[0];
   r.kinetic = p.kinetic;
   r.nsteps = nsteps;

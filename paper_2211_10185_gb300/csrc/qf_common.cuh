@@ -79,6 +79,7 @@ struct FftPassArgs {
   int v_real;
   R half_dtau;            // dtau / 2
   R dtau;
+  R dtau_lo;              // second part of dtau in the plane form (else unused)
   const double* scale;    // output scale (device scalar)
   double* partials;       // per-block FP64 sums when reducing
   int write_psi;          // 0: measure only (no write)

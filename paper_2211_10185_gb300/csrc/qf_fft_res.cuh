@@ -19,9 +19,7 @@
 // takes.  One step, before and now: N = 8: 7.0 / 1.6 us, 12: 11.2 / 2.1, 16: 13.0 / 2.2, 24:
 // 14.8 / 4.2, 32: 11.6 / 5.3.  At N = 48 (13.3 against 12.8 us) the 16 SMs of a cluster are too few.
 #pragma once
-#include <utility>
-
-#include "qf_fft_impl.cuh"
+#include "qf_fft_reg.cuh"
 
 namespace qf {
 
@@ -34,7 +32,7 @@ struct ResArgs {
   const double* scale;       // output scale of the first step
   const double* scale2;      // and of the others
   double* partials;          // kNumSums per block of the cluster when reducing
-  float tcoef, am2, half_dtau, dtau;
+  float tcoef, am2, half_dtau, dtau, dtau_lo;
   int* err;                  // set to 1 when a bounded wait ran out
   int kinetic, nsteps;
 };
@@ -99,113 +97,6 @@ __device__ __forceinline__ bool res_wait(unsigned long long* bar, unsigned parit
 __device__ __forceinline__ void res_expect(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(bytes)
                : "memory");
-}
-
-// ---- transforms of N points in a thread's registers ----------------------------------------
-// Packed complex FP32 sums: one instruction for both parts.
-__device__ __forceinline__ cpx<float> rc_add(cpx<float> a, cpx<float> b) {
-  cpx<float> r;
-  asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-__device__ __forceinline__ cpx<float> rc_sub(cpx<float> a, cpx<float> b) {
-  cpx<float> r;
-  asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-// cos and sin of 2 pi k / n, 0 <= k < n, from their Taylor series on [0, pi/4]
-constexpr double rc_series(double x, bool sine) {
-  double t = sine ? x : 1.0, s = t;
-  for (int i = sine ? 3 : 2; i < 24; i += 2) {
-    t *= -x * x / (double)(i * (i - 1));
-    s += t;
-  }
-  return s;
-}
-constexpr double rc_cos(int k, int n) {
-  const int o = 8 * k / n;                                  // octant
-  const double x = 6.283185307179586476925286766559 / n;
-  switch (o) {
-    case 0: return rc_series(x * k, false);
-    case 1: return rc_series(x * (n / 4.0 - k), true);
-    case 2: return -rc_series(x * (k - n / 4.0), true);
-    case 3: return -rc_series(x * (n / 2.0 - k), false);
-    case 4: return -rc_series(x * (k - n / 2.0), false);
-    case 5: return -rc_series(x * (3.0 * n / 4.0 - k), true);
-    case 6: return rc_series(x * (k - 3.0 * n / 4.0), true);
-    default: return rc_series(x * (n - k), false);
-  }
-}
-constexpr double rc_sin(int k, int n) { return rc_cos((k + n - n / 4) % n, n); }  // (n a multiple of 4)
-
-template <bool INV>
-__device__ __forceinline__ void rc_dft4(cpx<float>& x0, cpx<float>& x1, cpx<float>& x2, cpx<float>& x3) {
-  const cpx<float> a0 = rc_add(x0, x2), a1 = rc_sub(x0, x2), a2 = rc_add(x1, x3), d = rc_sub(x1, x3);
-  x0 = rc_add(a0, a2);
-  x2 = rc_sub(a0, a2);
-  const cpx<float> p = mk<float>(a1.x + d.y, a1.y - d.x), q = mk<float>(a1.x - d.y, a1.y + d.x);  // a1 -+ i d
-  x1 = INV ? q : p;
-  x3 = INV ? p : q;
-}
-template <bool INV>
-__device__ __forceinline__ void rc_dft3(cpx<float>& x0, cpx<float>& x1, cpx<float>& x2) {
-  const float h = 0.86602540378443864676f;  // sin(2 pi / 3)
-  const cpx<float> s = rc_add(x1, x2), d = rc_sub(x1, x2);
-  const cpx<float> t = mk<float>(fmaf(-0.5f, s.x, x0.x), fmaf(-0.5f, s.y, x0.y));
-  x0 = rc_add(x0, s);
-  const cpx<float> p = mk<float>(fmaf(h, d.y, t.x), fmaf(-h, d.x, t.y)), q = mk<float>(fmaf(-h, d.y, t.x), fmaf(h, d.x, t.y));
-  x1 = INV ? q : p;
-  x2 = INV ? p : q;
-}
-// a exp(-+ 2 pi i K / N)
-template <int K, int N, bool INV>
-__device__ __forceinline__ cpx<float> rc_rot(cpx<float> a) {
-  constexpr int k = K % N;
-  if constexpr (k == 0) return a;
-  else if constexpr (4 * k == N) return INV ? mk<float>(-a.y, a.x) : mk<float>(a.y, -a.x);
-  else if constexpr (2 * k == N) return mk<float>(-a.x, -a.y);
-  else if constexpr (4 * k == 3 * N) return INV ? mk<float>(a.y, -a.x) : mk<float>(-a.y, a.x);
-  else return rot<float, INV>(a, (float)rc_cos(k, N), (float)rc_sin(k, N));
-}
-template <int N, bool INV, int STRIDE>
-__device__ __forceinline__ void rc_dft(cpx<float>* x);
-// N = A B by decimation: A-point transforms over n1 of n = B n1 + n2, twiddles, B-point ones
-// over n2, output k = k1 + A k2.  x[STRIDE i] holds element i before and after.
-template <int N, int A, int B, bool INV, int STRIDE, int... I2, int... I1>
-__device__ __forceinline__ void rc_split(cpx<float>* x, std::integer_sequence<int, I2...>, std::integer_sequence<int, I1...>) {
-  (rc_dft<A, INV, STRIDE * B>(x + STRIDE * I2), ...);
-  auto twiddle = [&](auto n2c) {
-    constexpr int n2 = decltype(n2c)::value;
-    ((x[STRIDE * (B * I1 + n2)] = rc_rot<n2 * I1, N, INV>(x[STRIDE * (B * I1 + n2)])), ...);
-  };
-  (twiddle(std::integral_constant<int, I2>{}), ...);
-  (rc_dft<B, INV, STRIDE>(x + STRIDE * B * I1), ...);
-  cpx<float> y[N];
-#pragma unroll
-  for (int k1 = 0; k1 < A; ++k1)
-#pragma unroll
-    for (int k2 = 0; k2 < B; ++k2) y[k1 + A * k2] = x[STRIDE * (B * k1 + k2)];
-#pragma unroll
-  for (int k = 0; k < N; ++k) x[STRIDE * k] = y[k];
-}
-template <int N, bool INV, int STRIDE>
-__device__ __forceinline__ void rc_dft(cpx<float>* x) {
-  if constexpr (N == 2) {
-    const cpx<float> d = rc_sub(x[0], x[STRIDE]);
-    x[0] = rc_add(x[0], x[STRIDE]);
-    x[STRIDE] = d;
-  } else if constexpr (N == 3) {
-    rc_dft3<INV>(x[0], x[STRIDE], x[2 * STRIDE]);
-  } else if constexpr (N == 4) {
-    rc_dft4<INV>(x[0], x[STRIDE], x[2 * STRIDE], x[3 * STRIDE]);
-  } else {
-    constexpr int A = N == 8 ? 4 : N == 16 ? 4 : N == 32 ? 4 : 3, B = N / A;  // 12, 24: 3 x
-    rc_split<N, A, B, INV, STRIDE>(x, std::make_integer_sequence<int, B>{}, std::make_integer_sequence<int, A>{});
-  }
 }
 
 // The block's sums (THREADS need not fill its last warp) to out[0 .. kNumSums).
@@ -303,7 +194,7 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
     }
     const float sxy = sym[l] + sym[rank * P + s];
 #pragma unroll
-    for (int z = 0; z < N; ++z) v[z] = cscale<float>(v[z], kin_mult<float>(a.kinetic, sxy, sym[z], a.tcoef, a.am2));
+    for (int z = 0; z < N; ++z) v[z] = cscale<float>(v[z], kin_mult_acc(a.kinetic, sxy, sym[z], a.tcoef, a.am2));
 #pragma unroll kUnroll
     for (int ph = 0; ph < 3; ++ph) {  // z, y, x inverse
       rc_dft<N, true, 1>(v);
@@ -336,16 +227,8 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
     const float sc = t == 0 ? sc1 : sc2;
 #pragma unroll
     for (int x = 0; x < N; ++x) {
-      // d = 1 + dtau V/2; coef_B = 1/d; coef_A = (2 - d)/d
-      if constexpr (VREAL) {
-        const float d = 1.f + a.half_dtau * vr[x];
-        const cpx<float> num = cscale<float>(psi[x], 2.f - d) - cscale<float>(v[x], a.dtau);
-        psi[x] = cscale<float>(num, __fdividef(sc, d));
-      } else {
-        const cpx<float> d = mk<float>(1.f + a.half_dtau * vr[x], a.half_dtau * vi[x]);
-        const cpx<float> num = cmul<float>(mk<float>(2.f - d.x, -d.y), psi[x]) - cscale<float>(v[x], a.dtau);
-        psi[x] = cscale<float>(cmulc<float>(num, d), __fdividef(sc, d.x * d.x + d.y * d.y));
-      }
+      if constexpr (VREAL) psi[x] = reg_update(psi[x], v[x], vr[x], a.half_dtau, a.dtau, a.dtau_lo, sc);
+      else psi[x] = reg_update(psi[x], v[x], mk<float>(vr[x], vi[x]), a.half_dtau, a.dtau, a.dtau_lo, sc);
     }
   }
 #pragma unroll

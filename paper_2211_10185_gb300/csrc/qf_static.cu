@@ -143,7 +143,8 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
     r.a.tcoef = tcoef;
     r.a.am2 = am2;
     r.a.half_dtau = (float)(0.5 * dtau);
-    r.a.dtau = (float)dtau;
+    kinetic_dtau(n, dtau, kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3), tcoef, &r.a.dtau,
+                 &r.a.dtau_lo);
     r.a.kinetic = kinetic;
     r.a.nsteps = 1;
     if (launch_fft_res_static(n, r, !v_complex, sums != nullptr, st) != cudaSuccess) return QF_ECUDA;
