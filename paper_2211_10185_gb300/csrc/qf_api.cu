@@ -26,6 +26,8 @@ bool fft2_supported(int n);
 int fft2_final_blocks(int n);
 int fft2_measure_blocks(int n);
 bool plane_supported(int n);
+bool line_supported(int n);
+int line_final_blocks(int n);
 cudaError_t launch_fft2_group_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
 cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st);
 cudaError_t launch_bounded_wait_probe(int* err, cudaStream_t st);
@@ -195,6 +197,11 @@ struct qf_lattice {
 // The FFT step of this lattice runs the two-pass kernels.
 static bool uses_fft2(const qf_lattice* lat) {
   return lat->two_pass && lat->c64() && lat->kinetic != QF_KIN_FDTD && fft2_supported(lat->d.n);
+}
+
+// The four-pass FFT step of this lattice runs its z and x passes in the line form.
+static bool uses_line(const qf_lattice* lat) {
+  return lat->two_pass && lat->c64() && lat->kinetic > QF_KIN_FDTD && line_supported(lat->d.n);
 }
 
 // The FFT step of this lattice runs the resident kernel (many steps per launch).
@@ -543,8 +550,10 @@ static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduc
   p.write_psi = write ? 1 : 0;
   p.reduce = reduce ? 1 : 0;
   p.data = reinterpret_cast<cpx<R>*>(lat->tmp());
-  if constexpr (sizeof(R) == 4)
-    if (uses_fft2(lat) && plane_supported(lat->d.n)) form_dtau(lat, p.tcoef, &p.dtau, &p.dtau_lo);
+  if constexpr (sizeof(R) == 4) {
+    p.line = write && uses_line(lat) ? 1 : 0;
+    if (p.line || (uses_fft2(lat) && plane_supported(lat->d.n))) form_dtau(lat, p.tcoef, &p.dtau, &p.dtau_lo);
+  }
   return p;
 }
 
@@ -1544,7 +1553,8 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
       // complex-FP32 FDTD members of any size share a launch (the stencil kernel takes
       // each member's N from its block table); FFT members need the same plan (N)
       if (!M->c64() || (M->kinetic == QF_KIN_FDTD) != fdtd || (!fdtd && M->d.n != L->d.n)) continue;
-      if (!fdtd && (M->v_real != L->v_real || chk[q] != chk[k] || uses_fft2(M) != uses_fft2(L) || uses_res(M) != uses_res(L)))
+      if (!fdtd && (M->v_real != L->v_real || chk[q] != chk[k] || uses_fft2(M) != uses_fft2(L) || uses_res(M) != uses_res(L) ||
+                    uses_line(M) != uses_line(L)))
         continue;
       g.push_back(q);
       done[q] = 1;
@@ -1604,7 +1614,7 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
           const double* sq = M->pending_scale ? &M->sc()->scale[1] : &M->sc()->scale[2];
           fg.a[j] = fft_args<float>(M, M->psi(), true, chk[q], sq);
           fg.a[j].emit_next = 1;
-          nblk[q] = two ? fft2_final_blocks(n) : fft_final_blocks<float>(n);
+          nblk[q] = two ? fft2_final_blocks(n) : uses_line(M) ? line_final_blocks(n) : fft_final_blocks<float>(n);
           if (!M->xfwd_valid) {
             f0.a[f0.count] = fg.a[j];
             f0.a[f0.count].src = fg.a[j].psi;

@@ -84,6 +84,7 @@ struct FftPassArgs {
   double* partials;       // per-block FP64 sums when reducing
   int write_psi;          // 0: measure only (no write)
   int reduce;             // accumulate the kNumSums sums
+  int line;               // the step takes its line-form passes (qf_fft_line.cuh)
   int emit_next;          // final pass that writes psi': also write its forward x transform
                           // into data, so the next step can skip its first pass
 };

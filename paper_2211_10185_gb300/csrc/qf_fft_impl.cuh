@@ -694,6 +694,12 @@ int fft_tile_variant(int n);
 cudaError_t launch_fft_group_pass_t1(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
 cudaError_t launch_fft_group_pass_p1(int n, int variant, int pass, const FftGroup<float>& g, cudaStream_t st);
 
+// Line form of some passes of a step (qf_fft_line.cu).
+bool line_supported(int n);
+bool line_has_pass(int n, int pass);
+int line_final_blocks(int n);
+cudaError_t launch_line_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
+
 // Partial-sum rows of the reducing x pass for size n with tile variant V.
 template <typename R, int V>
 int fft_final_blocks_v(int n) {
@@ -714,6 +720,7 @@ int fft_final_blocks_v(int n) {
 template <typename R>
 cudaError_t launch_fft_group_pass(int n, int pass, const FftGroup<R>& g, cudaStream_t st, bool alt_plan) {
   if constexpr (sizeof(R) == 4) {
+    if (g.a[0].line && line_has_pass(n, pass)) return launch_line_pass(n, pass, g, st);
     int v = fft_tile_variant(n);
     if (!alt_plan) v &= 1;
     if (v >= 2) return launch_fft_group_pass_p1(n, v, pass, g, st);
@@ -758,7 +765,7 @@ template <typename R, int N>
 static cudaError_t single_pass_n(int pass, FftPassArgs<R> a, cpx<R>* tmp, cudaStream_t st, int* nfinal,
                                  bool alt_plan) {
   if constexpr (sizeof(R) == 4) {
-    if (nfinal) *nfinal = fft_final_blocks<R>(N);
+    if (nfinal) *nfinal = a.line ? line_final_blocks(N) : fft_final_blocks<R>(N);
     FftGroup<R> g;
     g.count = 1;
     g.a[0] = a;

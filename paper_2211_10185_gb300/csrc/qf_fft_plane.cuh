@@ -51,8 +51,9 @@ struct PlaneTable {
   constexpr PlaneTable() : w() {
     for (int g = 0; g < 4; ++g)
       for (int k = 0; k < N / 4; ++k) {
-        w[g * (N / 4) + k].x = (float)rc_cos(g * k % N, N);
-        w[g * (N / 4) + k].y = (float)-rc_sin(g * k % N, N);
+        const RcTwiddle t = rc_twiddle(g * k % N, N);
+        w[g * (N / 4) + k].x = t.c;
+        w[g * (N / 4) + k].y = -t.s;
       }
   }
 };
