@@ -4,7 +4,7 @@
 // One thread-block cluster holds a whole lattice and takes any number of steps per launch:
 // psi and V stay in registers, the transformed field in shared memory, and the two
 // redistributions of a step go through distributed shared memory.  Each of the cluster's C
-// blocks owns P = N / C z-planes; a thread transforms whole lines in registers:
+// blocks owns P = N / C z-planes; a thread (N = 32: four lanes) transforms a whole line:
 //   x forward, y forward on its planes  ->  column (kx, ky) to the block that owns ky
 //   z forward, T(k), z inverse          ->  column element z to the block that owns z
 //   y inverse, x inverse, update of psi in registers, and round again.
@@ -14,12 +14,13 @@
 // that a peer read last only after it has received everything that the peer sends once it
 // has read it.
 //
-// What bounds it: instruction issue and latency of few warps (N = 32: two per SM on 16 SMs).
+// What bounds it: instruction issue and latency of few warps (N = 32: eight per SM on 16 SMs; with a
+// line per thread, two per SM, 5.4 us a step, 6.3 with complex V and 6.0 with Eq. HK3).
 // The four-pass form needs four launches a step, each bound by the 2-3 us that any kernel
 // takes.  One step, before and now: N = 8: 7.0 / 1.6 us, 12: 11.2 / 2.1, 16: 13.0 / 2.2, 24:
-// 14.8 / 4.2, 32: 11.6 / 5.3.  At N = 48 (13.3 against 12.8 us) the 16 SMs of a cluster are too few.
+// 14.8 / 4.2, 32: 11.6 / 5.0.  At N = 48 (13.3 against 12.8 us) the 16 SMs of a cluster are too few.
 #pragma once
-#include "qf_fft_reg.cuh"
+#include "qf_fft_plane.cuh"
 
 namespace qf {
 
@@ -53,13 +54,15 @@ template <int N>
 struct ResG {
   static constexpr int C = N == 8 ? 2 : N == 12 ? 4 : N <= 24 ? 8 : 16;  // blocks per cluster
   static constexpr int P = N / C;
-  static constexpr int THREADS = P * N;  // one line each
-  // row pitch in elements: odd, so that lanes along a column and along a row both spread
-  // over all banks
-  static constexpr int NP = N + 1;
+  static constexpr int LANES = N == 32 ? 4 : 1;  // per line
+  static constexpr int THREADS = P * N * LANES;
+  // row pitch in elements: odd where a thread has a line, so that lanes along a column and
+  // along a row both spread over all banks; else the plane form's layout
+  static constexpr int NP = LANES == 1 ? N + 1 : N + 8;
   static constexpr int SLAB = N * NP;  // a plane [y][x], or a ky [z][kx]
+  static constexpr size_t TW = LANES == 1 ? 0 : 4 * (N / 4 + 2);
   static constexpr unsigned BYTES = P * N * N * 8;  // a block's share of a redistribution
-  static constexpr size_t SMEM = (size_t)2 * P * SLAB * 8 + N * 8 + 32 * kNumSums * 8;
+  static constexpr size_t SMEM = (TW + 2 * P * SLAB) * 8 + N * 8 + 32 * kNumSums * 8;
   static_assert(N % C == 0 && THREADS <= 1024, "resident geometry");
 };
 
@@ -124,6 +127,116 @@ __device__ __forceinline__ void res_block_sum(double (&s)[kNumSums], double* scr
   }
 }
 
+// N = 32: four lanes a line, as in the plane form (lane g holds the elements g + 4 m), so that a
+// block has 8 warps instead of 2.
+template <int N, bool VREAL, bool SUMS>
+__device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, float sc1, float sc2) {
+  using G = ResG<N>;
+  constexpr int P = G::P, E = N / 4, ST = N * 4;  // ST threads a slab
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* red_s = reinterpret_cast<double*>(smem_raw);
+  cpx<float>* tw_s = reinterpret_cast<cpx<float>*>(red_s + 32 * kNumSums);
+  cpx<float>* plane = tw_s + G::TW;
+  cpx<float>* cols = plane + P * G::SLAB;
+  float* sym = reinterpret_cast<float*>(cols + P * G::SLAB);
+  __shared__ alignas(8) unsigned long long bars[2];
+  const int tid = threadIdx.x, rank = blockIdx.x;
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&bars[i])) : "memory");
+      res_expect(&bars[i], G::BYTES);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  bool ok = true;
+  unsigned parity = 0;
+  plane_twiddles<N>(tw_s, G::THREADS);
+  for (int i = tid; i < N; i += G::THREADS) sym[i] = sym_g[i];
+  const int s = tid / ST, warp = (tid % ST) >> 5, lane = tid & 31;
+  const int xg = lane & 3, line = warp * 8 + (lane >> 2), cg = lane >> 3, col = warp * 8 + (lane & 7);
+  auto x_at = [&](int i) { return plane + s * G::SLAB + plane_idx<N>(line, i); };
+  auto y_at = [&](int i) { return plane + s * G::SLAB + plane_idx<N>(i, col); };
+  auto z_at = [&](int i) { return cols + s * G::SLAB + plane_idx<N>(i, col); };
+  auto slab_sync = [&] { asm volatile("bar.sync %0, %1;\n" ::"r"(1 + s), "n"(ST) : "memory"); };
+  const long long row = (((long long)rank * P + s) * N + line) * N + xg;
+  cpx<float> v[E], psi[E];
+  float vr[E], vi[VREAL ? 1 : E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    psi[m] = a.psi[row + 4 * m];
+    if constexpr (VREAL) {
+      vr[m] = reinterpret_cast<const float*>(a.v)[row + 4 * m];
+    } else {
+      const cpx<float> w = reinterpret_cast<const cpx<float>*>(a.v)[row + 4 * m];
+      vr[m] = w.x;
+      vi[m] = w.y;
+    }
+  }
+  cluster_sync();  // the tables are in place, and every block of the cluster is running
+  for (int t = 0; t < (SUMS ? 1 : a.nsteps); ++t) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = psi[m];
+    plane_line<N, false>(v, xg, tw_s, x_at);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < E; ++m) *x_at(xg + 4 * m) = v[m];
+    slab_sync();
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = *y_at(cg + 4 * m);
+    plane_line<N, false>(v, cg, tw_s, y_at);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int ky = cg + 4 * m;
+      st_cluster(cols + (ky % P) * G::SLAB + plane_idx<N>(rank * P + s, col), ky / P, v[m], &bars[0]);
+    }
+    ok = res_wait(&bars[0], parity, ok);
+    if (tid == 0) res_expect(&bars[0], G::BYTES);
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = *z_at(cg + 4 * m);
+    plane_line<N, false>(v, cg, tw_s, z_at);
+    const float sxy = sym[col] + sym[rank * P + s];
+#pragma unroll
+    for (int m = 0; m < E; ++m)
+      v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[cg + 4 * m], a.tcoef, a.am2));
+    plane_line<N, true>(v, cg, tw_s, z_at);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int z = cg + 4 * m;
+      st_cluster(plane + (z % P) * G::SLAB + plane_idx<N>(rank * P + s, col), z / P, v[m], &bars[1]);
+    }
+    ok = res_wait(&bars[1], parity, ok);
+    if (tid == 0) res_expect(&bars[1], G::BYTES);
+    parity ^= 1;
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = *y_at(cg + 4 * m);
+    plane_line<N, true>(v, cg, tw_s, y_at);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < E; ++m) *y_at(cg + 4 * m) = v[m];
+    slab_sync();
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = *x_at(xg + 4 * m);
+    plane_line<N, true>(v, xg, tw_s, x_at);
+    if constexpr (SUMS) {
+      CheckSums<float> sum;
+#pragma unroll
+      for (int m = 0; m < E; ++m) sum.add(psi[m], v[m], mk<float>(vr[m], VREAL ? 0.f : vi[VREAL ? 0 : m]));
+      double acc[kNumSums];
+      sum.to(acc);
+      res_block_sum<G::THREADS>(acc, red_s, a.partials + (long long)rank * kPartialStride);
+    }
+    const float sc = t == 0 ? sc1 : sc2;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      if constexpr (VREAL) psi[m] = reg_update(psi[m], v[m], vr[m], a.half_dtau, a.dtau, a.dtau_lo, sc);
+      else psi[m] = reg_update(psi[m], v[m], mk<float>(vr[m], vi[m]), a.half_dtau, a.dtau, a.dtau_lo, sc);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < E; ++m) a.psi[row + 4 * m] = psi[m];
+  if (!ok && a.err) atomicExch(a.err, 1);
+}
+
 template <int N, bool VREAL, bool SUMS>
 __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, float sc1, float sc2) {
   using G = ResG<N>;
@@ -168,8 +281,8 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
   cluster_sync();  // the symbol is in place, and every block of the cluster is running
   for (int t = 0; t < (SUMS ? 1 : a.nsteps); ++t) {
     // One copy of the transform's code a direction for the longer lines: with 2-3 warps per SM
-    // straight code of all six ran at the pace of the instruction cache (N = 32: 6.4 us a step,
-    // 5.3 so; N = 24: 4.4 and 4.2; N = 16: 2.2 straight, 2.4 so).
+    // straight code of all six ran at the pace of the instruction cache (N = 24: 4.4 us a step,
+    // 4.2 so; N = 16: 2.2 straight, 2.4 so).
     constexpr int kUnroll = N <= 16 ? 3 : 1;
 #pragma unroll
     for (int x = 0; x < N; ++x) v[x] = psi[x];
@@ -239,11 +352,13 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
 template <int N, bool VREAL, bool SUMS>
 __global__ void __launch_bounds__(ResG<N>::THREADS) fft_res_kernel(const __grid_constant__ ResGroup g) {
   const ResArgs& a = g.a[blockIdx.y];
-  res_body<N, VREAL, SUMS>(a, a.symbol, (float)*a.scale, (float)*a.scale2);
+  if constexpr (ResG<N>::LANES == 4) res_body4<N, VREAL, SUMS>(a, a.symbol, (float)*a.scale, (float)*a.scale2);
+  else res_body<N, VREAL, SUMS>(a, a.symbol, (float)*a.scale, (float)*a.scale2);
 }
 template <int N, bool VREAL, bool SUMS>
 __global__ void __launch_bounds__(ResG<N>::THREADS) fft_res_static_kernel(const __grid_constant__ ResStatic g) {
-  res_body<N, VREAL, SUMS>(g.a, g.sym, (float)g.out_scale, (float)g.out_scale);
+  if constexpr (ResG<N>::LANES == 4) res_body4<N, VREAL, SUMS>(g.a, g.sym, (float)g.out_scale, (float)g.out_scale);
+  else res_body<N, VREAL, SUMS>(g.a, g.sym, (float)g.out_scale, (float)g.out_scale);
 }
 
 // nsteps steps of every member of g (one lattice size, one kind of potential) in one launch;
