@@ -416,7 +416,12 @@ __device__ __forceinline__ void fft_x_body(const FftPassArgs<R>& a, const int bi
           // d = 1 + dtau V/2; coef_B = 1/d; coef_A = (2 - d)/d (FP32: the fast hardware
           // division, a few ulp; FP64: correctly rounded)
           const cpx<R> vi = vat(i);
-          if constexpr (VREAL) {
+          if constexpr (VREAL && sizeof(R) == 8) {
+            // the reciprocal from the lattice's table: coef_A = 2/d - 1
+            const R is = a.inv[base + e_out<N, S - 1, PL>(g, b, r)] * sc;
+            const R ca = fma(R(2), is, -sc), cb = a.dtau * is;
+            v[i] = mk<R>(fma(ca, pv[i].x, -(cb * v[i].x)), fma(ca, pv[i].y, -(cb * v[i].y)));
+          } else if constexpr (VREAL) {
             const R d = R(1) + a.half_dtau * vi.x;
             const cpx<R> num = cscale<R>(pv[i], R(2) - d) - cscale<R>(v[i], a.dtau);
             if constexpr (sizeof(R) == 4) v[i] = cscale<R>(num, __fdividef(sc, d));

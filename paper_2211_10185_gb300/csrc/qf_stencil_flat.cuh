@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kFlatThreads) stencil_flat_kernel(const __grid
   const bool hxm = live && x > 1, hxp = live && x + 1 < n, hym = live && y > 1, hyp = live && y + 1 < n;
   const cpx<R> zero = mk<R>(R(0), R(0));
   const cpx<R>* __restrict__ in = a.in;
-  const R sc = R(*a.scale);
+  const R sc = R(*a.scale), c26 = R(2) - R(6) * a.kd;
   CheckSums<R> cs;
   long long site = (long long)z0 * n2 + p;
   cpx<R> zm = zero, c = zero;
@@ -173,10 +173,22 @@ __global__ void __launch_bounds__(kFlatThreads) stencil_flat_kernel(const __grid
       if (hxp) xp = in[site + 1];
       if (hym) ym = in[site - n];
       if (hyp) yp = in[site + n];
-      if (live) vv = a.v_real ? mk<R>(reinterpret_cast<const R*>(a.v)[site], R(0)) : reinterpret_cast<const cpx<R>*>(a.v)[site];
+      if (live && (sizeof(R) == 4 || !a.inv || a.reduce)) vv = a.v_real ? mk<R>(reinterpret_cast<const R*>(a.v)[site], R(0)) : reinterpret_cast<const cpx<R>*>(a.v)[site];
     }
     if (live && up) {
-      const cpx<R> lap = lap_of<R>(c, six_sum<R>(xm, xp, ym, yp, zm, zp));
+      const cpx<R> nbs = six_sum<R>(xm, xp, ym, yp, zm, zp);
+      if constexpr (sizeof(R) == 8) {
+        if (a.inv && a.write_psi && !a.reduce) {
+          // psi' = sc ((2 - 6 kd) / d - 1) psi + sc kd / d nbs: 17 FP64 operations a site, 1/d from
+          // the lattice's table, where lap, the update and the division take 29
+          const R is = a.inv[site] * sc, ca = fma(c26, is, -sc), cb = a.kd * is;
+          a.out[site] = mk<R>(fma(ca, c.x, cb * nbs.x), fma(ca, c.y, cb * nbs.y));
+          zm = c;
+          c = zp;
+          continue;
+        }
+      }
+      const cpx<R> lap = lap_of<R>(c, nbs);
       if (a.reduce) cs.add(c, mk<R>(mul_rn<R>(-a.kcoef, lap.x), mul_rn<R>(-a.kcoef, lap.y)), vv);
       if (a.write_psi) a.out[site] = fdtd_update<R>(c, lap, vv, a.v_real != 0, a.half_dtau, a.kd, sc);
     } else if (in_plane && a.write_psi) {
