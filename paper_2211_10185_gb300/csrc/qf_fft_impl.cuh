@@ -75,16 +75,23 @@ constexpr int largest_divisor_le(int n, int cap) {
   return best;
 }
 
-// Tile geometry of the four-pass kernels.  Bit 0 of V: 0 = about 4096 (FP32) / 2048
+// Tile geometry of the four-pass kernels.  Bit 0 of V: 0 = about 4096 (FP32) / fp64_target
 // (FP64) elements per tile, y/z tiles up to 16 (8) contiguous columns wide; 1 = half the
 // tile and half the width (more, smaller blocks per SM).  Bit 1: the radix plan (PLAN).
-// The autotuner picks V per N.
+// The autotuner picks V per N.  FP64 passes are bound by the FP64 pipe (2 fused multiply-adds per
+// clock and SM), so what counts is that the blocks spread evenly over the SMs: 8 lines or
+// columns a block (a warp; 32 where a thread has a whole line) at the sizes where 2048 elements
+// a block left SMs idle or a thin last wave.  One step of Eq. HK3 with 2048 elements / so: N = 32:
+// 67.5 / 36.5 us, 96: 303 / 261; no gain at 64 (78.8 / 79.7) and 128 (588 / 602).
+constexpr int fp64_target(int n) {
+  return n == 32 || n == 48 || n == 96 || n == 192 ? 8 * n : n == 8 || n == 16 || n == 24 ? 32 * n : 2048;
+}
 template <typename R, int N, int V = 0>
 struct Geom {
   static constexpr int PLAN = V >> 1;
   static constexpr int EPT = plan_ept(N, PLAN);
   static constexpr int S = plan_stages(N, PLAN);
-  static constexpr int TARGET = (sizeof(R) == 4 ? 4096 : 2048) >> (V & 1);  // elements per tile
+  static constexpr int TARGET = (sizeof(R) == 4 ? 4096 : fp64_target(N)) >> (V & 1);  // elements per tile
   // x pass: LC whole lines per block
   static constexpr int LC = largest_divisor_le(N * N, TARGET / N > 0 ? TARGET / N : 1);
   static constexpr int TL = N / EPT;                       // threads per line
