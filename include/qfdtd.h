@@ -104,8 +104,9 @@ typedef struct {
   size_t workspace_bytes;
   int64_t launches;   /* kernels this handle has launched so far                     */
   int temporal_block; /* FDTD steps fused per pass (qf_set_temporal_blocking)         */
-  int fft_passes;     /* HBM passes of a steady-state FFT step: 2 (N = 128 or 256
-                         complex FP32, qf_use_two_pass_fft) or 4; 0 for FDTD          */
+  int fft_passes;     /* launches of a steady-state FFT step: 2 (complex FP32 with N = 48,
+                         64, 96, 128 or 256, qf_use_two_pass_fft) or 4 (also reported for
+                         resident lattices, N <= 32); 0 for FDTD                      */
   int64_t field_exp2; /* the stored live field is 2^field_exp2 times the one
                          qf_get_wavefunction returns (see qf_step_n)                  */
 } qf_info;
@@ -219,18 +220,20 @@ qf_status qf_momentum_distribution(qf_lattice* lat, int slot, double* p, double*
 qf_status qf_use_graphs(qf_lattice* lat, int enable);
 
 /* Form of the FFT step (no counterpart in the paper; the paper's FFTW transforms are
- * replaced by GPU passes).  enable != 0, the default: complex-FP32 lattices with N = 128
- * or 256 run a steady-state step in two passes over HBM (the y transform split
+ * replaced by GPU passes).  enable != 0, the default: complex-FP32 lattices take the
+ * fastest form of their size: N <= 32 many steps per launch with the lattice resident in a
+ * thread-block cluster (8, 12, 16, 24, 32), N = 48, 64 and 96 two launches per step, one of
+ * them per z-plane, N = 128 and 256 two passes over HBM (the y transform split
  * (N/16) x 16 four-step fashion between the two passes; the scratch field holds a
- * blocked layout), other lattices in four.  enable == 0 selects the four-pass form for
- * N = 128 and 256 too.  Both
+ * blocked layout), N = 192 and 512 four passes with warp-wide lines, others plain four
+ * passes.  enable == 0 selects the plain four-pass form for every size.  All
  * compute the same step to rounding; switching discards the scratch field's contents and
  * any captured graphs. */
 qf_status qf_use_two_pass_fft(qf_lattice* lat, int enable);
 
 /* Tile and radix-plan choice of the complex-FP32 four-pass FFT kernels for lattice size n
- * (no counterpart in the paper; every size, N = 128 and 256 when their four-pass form is
- * selected).  Variant 0 tiles about 4096 elements per block with up to 16 contiguous
+ * (no counterpart in the paper; every size, where the lattice takes the four-pass form:
+ * qf_use_two_pass_fft).  Variant 0 tiles about 4096 elements per block with up to 16 contiguous
  * columns; variant 1 half of both (more, smaller blocks per SM); the two compute the same
  * transforms (the fields agree bitwise; reductions may differ in their last bits).
  * Variants 2 and 3 are variants 0 and 1 with the size's second radix plan (a radix-16
@@ -246,8 +249,8 @@ qf_status qf_get_fft_tiles(int n, int* variant);
 /* Temporal blocking of the FDTD step (the step of Sec. 2 with the Eq. HK0 term; no
  * counterpart in the paper).  k = 2, the default: on complex-FP32 lattices qf_step_n
  * runs two consecutive steps with no check at either and no snapshot after the first as
- * one pass over HBM (psi_t and V read once, psi_{t+2} written once, psi_{t+1} kept in
- * shared memory).  The fields are bitwise those of two single steps.  Requires the live
+ * one pass over HBM (psi_t and V read once, psi_{t+2} written once, psi_{t+1} kept on
+ * chip).  The fields are bitwise those of two single steps.  Requires the live
  * field to be zero on the Dirichlet planes, which holds after any FDTD step; the first
  * step after qf_set_wavefunction always runs alone.  k = 1 runs every step alone.  Other
  * precisions and kinetic terms ignore the setting.  QF_EINVAL unless k is 1 or 2. */
@@ -314,7 +317,7 @@ qf_status qf_fft_step_static(int n, double a, int kinetic, double mass, double d
  * form groups, and each pass of a group is a single kernel launch over all its members
  * (up to 48 per launch): FDTD lattices of any sizes together (the stencil launch maps
  * its blocks to members through a table), FFT lattices of equal N, real/complex V and
- * check status; FP64 lattices run their own launches.  Every member computes
+ * check status (a launch takes several steps where a lone lattice's does); FP64 lattices run their own launches.  Every member computes
  * exactly what qf_step_n computes for it alone (same kernels, same blocks, same
  * reduction order), so its results do not depend on the other members.  A batch holds
  * no device memory; members keep their own workspaces.  During qf_batch_step all
