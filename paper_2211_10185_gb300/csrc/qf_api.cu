@@ -1,7 +1,8 @@
 // C ABI of libqfdtd (declared in include/qfdtd.h): lattice handles over a caller-owned
 // device workspace, the step loop with its checks and snapshots, Gram-Schmidt excited
 // states and parity projection.  Every arithmetic step on fields runs in the kernels of
-// qf_fft_impl.cuh (four-pass FFT step), qf_fft2.cuh (two-pass step, N = 128 and 256),
+// qf_fft_impl.cuh (four-pass FFT step), qf_fft_res.cuh, qf_fft_plane.cuh, qf_fft2.cuh and
+// qf_fft_line.cuh (its forms by lattice size),
 // qf_stencil_flat.cuh / qf_stencil_tb.cuh (FDTD steps) and qf_fields.cu; this file only
 // sequences them.
 #include <math.h>
@@ -161,7 +162,7 @@ struct qf_lattice {
   // the Dirichlet planes (it is after any FDTD step), which the two-step kernel needs
   int tblock = 2;
   bool clean = false;
-  // N = 128 and 256 complex-FP32 FFT steps in two passes over HBM (qf_fft2.cuh) instead of four;
+  // complex-FP32 FFT steps in the form of their size instead of the four-pass one;
   // the scratch field then holds the four-step layout, so switching drops xfwd_valid
   bool two_pass = true;
   std::string err;
@@ -194,7 +195,7 @@ struct qf_lattice {
   bool c64() const { return d.prec == QF_PREC_C64; }
 };
 
-// The FFT step of this lattice runs the two-pass kernels.
+// The FFT step of this lattice runs two launches (plane or split form).
 static bool uses_fft2(const qf_lattice* lat) {
   return lat->two_pass && lat->c64() && lat->kinetic != QF_KIN_FDTD && fft2_supported(lat->d.n);
 }

@@ -1,5 +1,6 @@
-// The two-pass FFT step for N = 256 (the N = 128 instantiation is in qf_fft2_n128.cu, a
-// translation unit of its own so that the two compile in parallel), and the size dispatch.
+// The split two-pass FFT step for N = 256 (the N = 128 instantiation is in qf_fft2_n128.cu, a
+// translation unit of its own so that the two compile in parallel), and the size dispatch of
+// the two-launch forms.
 #include "qf_fft2_launch.cuh"
 
 namespace qf {

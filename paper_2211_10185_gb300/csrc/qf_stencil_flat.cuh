@@ -99,11 +99,12 @@ __device__ __forceinline__ cpx<R> fdtd_update(cpx<R> c, cpx<R> lap, cpx<R> v, bo
 // lane is lost on sizes that 32 does not divide) and marches through zc planes with the
 // z-neighbours in registers; the four in-plane neighbours come through L1 and L2.  Nothing is
 // staged in shared memory.  What bounds it: the FP64 pipe in complex FP64 (2 fused
-// multiply-adds per clock and SM, about 29 per site), HBM and L2 in complex FP32, latency on
-// small lattices, which need as many blocks as they have rows: the 32 x 32 tiles of 8 planes
-// used before left all but 4 SMs idle at N = 32.  One step, before and now: complex FP64
-// N = 32: 69 / 4.5 us, 64: 71 / 16, 128: 133 / 117, 192: 385 / 363; complex FP32 N = 32: 23 /
-// 10 us, 250: 112 / 109, 512: 783 / 786 (bracketed by events).
+// multiply-adds per clock and SM: 17 per site with the reciprocal table of a real V, 29
+// without), HBM and L2 in complex FP32, latency on small lattices, which need as many blocks as
+// they have rows: the 32 x 32 tiles of 8 planes used before left all but 4 SMs idle at N = 32.
+// One step, before and now (in brackets: without the table): complex FP64 N = 32: 69 / 3.6 (4.5)
+// us, 64: 71 / 12 (16), 128: 133 / 88 (117); complex FP32 N = 32: 23 / 10 us, 250: 112 / 109,
+// 512: 783 / 786 (bracketed by events).
 constexpr int kFlatThreads = 128;
 
 // Members of one launch may have different lattice sizes: member i runs
