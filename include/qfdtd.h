@@ -105,8 +105,8 @@ typedef struct {
   int64_t launches;   /* kernels this handle has launched so far                     */
   int temporal_block; /* FDTD steps fused per pass (qf_set_temporal_blocking)         */
   int fft_passes;     /* launches of a steady-state FFT step: 2 (complex FP32 with N = 48,
-                         64, 96, 128 or 256, qf_use_two_pass_fft) or 4 (also reported for
-                         resident lattices, N <= 32); 0 for FDTD                      */
+                         64, 128 or 256, or N = 96 where qf_use_two_pass_fft asked for it)
+                         or 4 (also reported for resident lattices, N <= 32); 0 for FDTD */
   int64_t field_exp2; /* the stored live field is 2^field_exp2 times the one
                          qf_get_wavefunction returns (see qf_step_n)                  */
 } qf_info;
@@ -220,13 +220,14 @@ qf_status qf_momentum_distribution(qf_lattice* lat, int slot, double* p, double*
 qf_status qf_use_graphs(qf_lattice* lat, int enable);
 
 /* Form of the FFT step (no counterpart in the paper; the paper's FFTW transforms are
- * replaced by GPU passes).  enable != 0, the default: complex-FP32 lattices take the
+ * replaced by GPU passes).  enable != 0: complex-FP32 lattices take the
  * fastest form of their size: N <= 32 many steps per launch with the lattice resident in a
  * thread-block cluster (8, 12, 16, 24, 32), N = 48, 64 and 96 two launches per step, one of
  * them per z-plane, N = 128 and 256 two passes over HBM (the y transform split
  * (N/16) x 16 four-step fashion between the two passes; the scratch field holds a
  * blocked layout), N = 192 and 512 four passes with warp-wide lines, others plain four
- * passes.  enable == 0 selects the plain four-pass form for every size.  All
+ * passes.  enable == 0 selects the plain four-pass form for every size.  The default is
+ * enable != 0 for every size but N = 96, which takes the plain four-pass form.  All
  * compute the same step to rounding; switching discards the scratch field's contents and
  * any captured graphs. */
 qf_status qf_use_two_pass_fft(qf_lattice* lat, int enable);

@@ -162,8 +162,9 @@ struct qf_lattice {
   // the Dirichlet planes (it is after any FDTD step), which the two-step kernel needs
   int tblock = 2;
   bool clean = false;
-  // complex-FP32 FFT steps in the form of their size instead of the four-pass one;
-  // the scratch field then holds the four-step layout, so switching drops xfwd_valid
+  // complex-FP32 FFT steps in the form of their size instead of the four-pass one: the default of
+  // the size (default_form), or what qf_use_two_pass_fft asked for.  The scratch field's layout
+  // depends on the form, so switching drops xfwd_valid
   bool two_pass = true;
   std::string err;
   // launch accounting and optional CUDA-event timing per kernel kind
@@ -210,6 +211,13 @@ static bool uses_res(const qf_lattice* lat) {
   return lat->two_pass && lat->c64() && lat->kinetic > QF_KIN_FDTD && res_supported(lat->d.n) &&
          fft_res_blocks(lat->d.n) > 0;
 }
+
+// Sizes whose form is the default.  N = 96 takes the four-pass form unless asked for: the plane
+// form's field and energy (a step in 17.9 us against 25.1) differ from the four-pass form's by the
+// roundings of both, 1e-7 of <T> at the start field and up to 1e-6 after 64 steps (the plane
+// form 1e-7 from 64-bit arithmetic, the four-pass form 8e-7), which is 1e-4 of E where <T> and <V>
+// nearly cancel; and at this size it holds 96 lines of two fields in registers and spills.
+static bool default_form(int n) { return n != 96; }
 
 static void drop_graphs(qf_lattice* lat) {
   for (auto& g : lat->graphs) cudaGraphExecDestroy(g.exec);
@@ -290,6 +298,7 @@ extern "C" qf_status qf_create_lattice(const qf_lattice_desc* desc, void* dev_ws
   lat->ws = static_cast<char*>(dev_ws);
   lat->st = static_cast<cudaStream_t>(stream);
   lat->sites = (long long)desc->n * desc->n * desc->n;
+  lat->two_pass = default_form(desc->n);
   cudaError_t e = cudaMemsetAsync(lat->ws, 0, L.total, lat->st);
   if (e == cudaSuccess) {
     DevScalars init{};

@@ -147,7 +147,7 @@ class Lattice:
         _check(self.h, self.lib.qf_use_graphs(self.h, int(bool(enable))), "qf_use_graphs")
 
     def use_two_pass_fft(self, enable: bool = True):
-        """Two HBM passes per FFT step for N = 128 and 256 complex FP32 (default) or four."""
+        """The complex-FP32 FFT step in the form of its size (default, N = 96 apart) or in four passes."""
         _check(self.h, self.lib.qf_use_two_pass_fft(self.h, int(bool(enable))), "qf_use_two_pass_fft")
 
     def set_temporal_blocking(self, k: int):
