@@ -309,7 +309,10 @@ qf_status qf_profile_read(qf_lattice* lat, qf_kernel_stat* out, int max, int* co
  * The first call on a device looks up the array's device address; make that first call
  * before any stream capture.  All calls share the one array and it keeps the previous
  * call's contents (each call rewrites everything it reads), so calls whose GPU work
- * overlaps -- on different streams or from different threads on one device -- race. */
+ * overlaps -- on different streams or from different threads on one device -- race.
+ * The step of n <= 32 runs in one cluster of blocks that wait for one another, each wait with
+ * a limit; should one run out, this call, which does not wait for its kernels, cannot say so:
+ * sites of psi, and <psi|psi> in sums, are NaN then. */
 qf_status qf_fft_step_static(int n, double a, int kinetic, double mass, double dtau, void* psi, const void* v,
                              int v_complex, double out_scale, double* sums, void* cuda_stream);
 
@@ -385,8 +388,9 @@ const char* qf_last_error(const qf_lattice* lat);
 /* Self-test of the bounded device waits (no counterpart in the paper; failure
  * detection).  Launches, on the handle's stream, a kernel whose wait on a
  * shared-memory barrier can never complete; the wait gives up after its iteration limit
- * (about a second), the kernel records the failure and returns, and this call returns
- * QF_ETIMEOUT with the context still usable.  QF_OK would mean the limit did not work. */
+ * (about a second), the kernel records the failure and returns; then resident FFT steps of
+ * 8^3 sites in the handle's scratch field whose waits are given no time.  This call returns
+ * QF_ETIMEOUT with the context still usable.  QF_OK would mean that a limit did not work. */
 qf_status qf_selftest_bounded_wait(qf_lattice* lat);
 
 /* Library version string. */

@@ -606,6 +606,7 @@ static ResArgs res_args(qf_lattice* lat, const double* scale, int nsteps) {
   r.err = &lat->sc()->err[0];
   r.kinetic = p.kinetic;
   r.nsteps = nsteps;
+  r.spin = kResSpin;
   return r;
 }
 
@@ -1448,7 +1449,29 @@ extern "C" qf_status qf_selftest_bounded_wait(qf_lattice* lat) {
   int err = 0;
   QF_CUDA(lat, cudaMemcpyAsync(&err, flag, sizeof(int), cudaMemcpyDeviceToHost, lat->st));
   QF_CUDA(lat, cudaStreamSynchronize(lat->st));
-  return err ? QF_ETIMEOUT : QF_OK;
+  if (!err || fft_res_blocks(8) == 0) return err ? QF_ETIMEOUT : QF_OK;
+  // resident steps of an 8^3 lattice in the scratch field whose waits are given no time: they
+  // must end, set the flag and leave NaN
+  ResGroup g{};
+  g.count = 1;
+  ResArgs& r = g.a[0];
+  r.psi = static_cast<cpx<float>*>(lat->tmp());
+  r.v = lat->ws + lat->L.v;
+  r.symbol = reinterpret_cast<const float*>(lat->ws + lat->L.sym);
+  r.scale = r.scale2 = &lat->sc()->scale[0];
+  r.partials = lat->partials();
+  r.err = flag;
+  r.kinetic = QF_KIN_FFT_NAIVE;
+  r.nsteps = 3;
+  r.spin = 0;
+  lat->xfwd_valid = false;
+  float site[2] = {0, 0};
+  QF_CUDA(lat, cudaMemsetAsync(flag, 0, sizeof(int), lat->st));
+  QF_CUDA(lat, launch_fft_res(8, g, true, false, lat->st));
+  QF_CUDA(lat, cudaMemcpyAsync(&err, flag, sizeof(int), cudaMemcpyDeviceToHost, lat->st));
+  QF_CUDA(lat, cudaMemcpyAsync(site, lat->tmp(), sizeof(site), cudaMemcpyDeviceToHost, lat->st));
+  QF_CUDA(lat, cudaStreamSynchronize(lat->st));
+  return err && isnan(site[0]) && isnan(site[1]) ? QF_ETIMEOUT : QF_OK;
 }
 
 // ------------------------------------------------------------------------------------

@@ -14,6 +14,12 @@
 // that a peer read last only after it has received everything that the peer sends once it
 // has read it.
 //
+// A wait is bounded.  A thread whose wait runs out sends nothing more and re-arms no barrier, but
+// keeps to the block barriers; without its share no later redistribution completes, so every
+// other thread's next wait runs out too and a launch ends after two limits.  Such a thread
+// stores NaN for its sites (the allocation-free step has no other way to say so), sets the
+// error flag, and holds its block until no thread of the cluster can store into it any more.
+//
 // What bounds it: instruction issue and latency of few warps (N = 32: eight per SM on 16 SMs; with a
 // line per thread, two per SM, 5.4 us a step, 6.3 with complex V and 6.0 with Eq. HK3).
 // The four-pass form needs four launches a step, each bound by the 2-3 us that any kernel
@@ -36,6 +42,7 @@ struct ResArgs {
   float tcoef, am2, half_dtau, dtau, dtau_lo;
   int* err;                  // set to 1 when a bounded wait ran out
   int kinetic, nsteps;
+  unsigned spin;             // tries of a wait (kResSpin)
 };
 struct ResGroup {
   int count;
@@ -47,6 +54,10 @@ struct ResStatic {
   float sym[32];
   double out_scale;
 };
+
+// Tries before a wait runs out, and for what may still be under way after that (a store between
+// the blocks of a cluster takes microseconds, a try tens of nanoseconds at least).
+constexpr unsigned kResSpin = 1u << 24, kResDrain = 1u << 16;
 
 constexpr bool res_supported(int n) { return n == 8 || n == 12 || n == 16 || n == 24 || n == 32; }
 
@@ -85,9 +96,9 @@ __device__ __forceinline__ void st_cluster(cpx<float>* p, int rank, cpx<float> v
 }
 // Bounded wait for phase `parity` of the block's own barrier (acquires what the cluster's
 // blocks stored); after a time-out it returns false at once for the rest of the launch.
-__device__ __forceinline__ bool res_wait(unsigned long long* bar, unsigned parity, bool ok) {
+__device__ __forceinline__ bool res_wait(unsigned long long* bar, unsigned parity, bool ok, unsigned spin) {
   const unsigned b = (unsigned)__cvta_generic_to_shared(bar);
-  for (unsigned it = 0; ok && it < (1u << 24); ++it) {
+  for (unsigned it = 0; ok && it < spin; ++it) {
     unsigned done;
     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
                  : "=r"(done)
@@ -100,6 +111,17 @@ __device__ __forceinline__ bool res_wait(unsigned long long* bar, unsigned parit
 __device__ __forceinline__ void res_expect(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(bytes)
                : "memory");
+}
+
+// End of a thread whose wait ran out (see above).  Every thread that has not exited has sent all it
+// will once it has arrived here (and one that has exited counts as arrived: its block had
+// received everything).  What is still under way counts on the phases that the block's barriers
+// are in: of the two waits on each, one is for the phase before and returns at once.
+__device__ __forceinline__ void res_close(bool ok, int* err, unsigned long long* bars) {
+  if (ok) return;
+  if (err) atomicExch(err, 1);
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+  for (int i = 0; i < 4; ++i) res_wait(&bars[i >> 1], i & 1, true, kResDrain);
 }
 
 // The block's sums (THREADS need not fill its last warp) to out[0 .. kNumSums).
@@ -184,13 +206,15 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = *y_at(cg + 4 * m);
     plane_line<N, false>(v, cg, tw_s, y_at);
+    if (ok) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-      const int ky = cg + 4 * m;
-      st_cluster(cols + (ky % P) * G::SLAB + plane_idx<N>(rank * P + s, col), ky / P, v[m], &bars[0]);
+      for (int m = 0; m < E; ++m) {
+        const int ky = cg + 4 * m;
+        st_cluster(cols + (ky % P) * G::SLAB + plane_idx<N>(rank * P + s, col), ky / P, v[m], &bars[0]);
+      }
     }
-    ok = res_wait(&bars[0], parity, ok);
-    if (tid == 0) res_expect(&bars[0], G::BYTES);
+    ok = res_wait(&bars[0], parity, ok, a.spin);
+    if (ok && tid == 0) res_expect(&bars[0], G::BYTES);
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = *z_at(cg + 4 * m);
     plane_line<N, false>(v, cg, tw_s, z_at);
@@ -199,13 +223,15 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
     for (int m = 0; m < E; ++m)
       v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[cg + 4 * m], a.tcoef, a.am2));
     plane_line<N, true>(v, cg, tw_s, z_at);
+    if (ok) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-      const int z = cg + 4 * m;
-      st_cluster(plane + (z % P) * G::SLAB + plane_idx<N>(rank * P + s, col), z / P, v[m], &bars[1]);
+      for (int m = 0; m < E; ++m) {
+        const int z = cg + 4 * m;
+        st_cluster(plane + (z % P) * G::SLAB + plane_idx<N>(rank * P + s, col), z / P, v[m], &bars[1]);
+      }
     }
-    ok = res_wait(&bars[1], parity, ok);
-    if (tid == 0) res_expect(&bars[1], G::BYTES);
+    ok = res_wait(&bars[1], parity, ok, a.spin);
+    if (ok && tid == 0) res_expect(&bars[1], G::BYTES);
     parity ^= 1;
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = *y_at(cg + 4 * m);
@@ -223,6 +249,7 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
       for (int m = 0; m < E; ++m) sum.add(psi[m], v[m], mk<float>(vr[m], VREAL ? 0.f : vi[VREAL ? 0 : m]));
       double acc[kNumSums];
       sum.to(acc);
+      if (!ok) acc[0] = __longlong_as_double(-1LL);
       res_block_sum<G::THREADS>(acc, red_s, a.partials + (long long)rank * kPartialStride);
     }
     const float sc = t == 0 ? sc1 : sc2;
@@ -232,9 +259,10 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
       else psi[m] = reg_update(psi[m], v[m], mk<float>(vr[m], vi[m]), a.half_dtau, a.dtau, a.dtau_lo, sc);
     }
   }
+  const float nan = __int_as_float(-1);
 #pragma unroll
-  for (int m = 0; m < E; ++m) a.psi[row + 4 * m] = psi[m];
-  if (!ok && a.err) atomicExch(a.err, 1);
+  for (int m = 0; m < E; ++m) a.psi[row + 4 * m] = ok ? psi[m] : mk<float>(nan, nan);
+  res_close(ok, a.err, bars);
 }
 
 template <int N, bool VREAL, bool SUMS>
@@ -296,11 +324,13 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
 #pragma unroll
         for (int y = 0; y < N; ++y) v[y] = ycol[y * NP];
       } else if (ph == 1) {
+        if (ok) {
 #pragma unroll
-        for (int ky = 0; ky < N; ++ky)
-          st_cluster(cols + (ky % P) * G::SLAB + (rank * P + s) * NP + l, ky / P, v[ky], &bars[0]);
-        ok = res_wait(&bars[0], parity, ok);
-        if (tid == 0) res_expect(&bars[0], G::BYTES);
+          for (int ky = 0; ky < N; ++ky)
+            st_cluster(cols + (ky % P) * G::SLAB + (rank * P + s) * NP + l, ky / P, v[ky], &bars[0]);
+        }
+        ok = res_wait(&bars[0], parity, ok, a.spin);
+        if (ok && tid == 0) res_expect(&bars[0], G::BYTES);
 #pragma unroll
         for (int z = 0; z < N; ++z) v[z] = zcol[z * NP];
       }
@@ -312,11 +342,13 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
     for (int ph = 0; ph < 3; ++ph) {  // z, y, x inverse
       rc_dft<N, true, 1>(v);
       if (ph == 0) {
+        if (ok) {
 #pragma unroll
-        for (int z = 0; z < N; ++z)
-          st_cluster(plane + (z % P) * G::SLAB + (rank * P + s) * NP + l, z / P, v[z], &bars[1]);
-        ok = res_wait(&bars[1], parity, ok);
-        if (tid == 0) res_expect(&bars[1], G::BYTES);
+          for (int z = 0; z < N; ++z)
+            st_cluster(plane + (z % P) * G::SLAB + (rank * P + s) * NP + l, z / P, v[z], &bars[1]);
+        }
+        ok = res_wait(&bars[1], parity, ok, a.spin);
+        if (ok && tid == 0) res_expect(&bars[1], G::BYTES);
         parity ^= 1;
 #pragma unroll
         for (int y = 0; y < N; ++y) v[y] = ycol[y * NP];
@@ -335,6 +367,7 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
       for (int x = 0; x < N; ++x) sum.add(psi[x], v[x], mk<float>(vr[x], VREAL ? 0.f : vi[VREAL ? 0 : x]));
       double acc[kNumSums];
       sum.to(acc);
+      if (!ok) acc[0] = __longlong_as_double(-1LL);
       res_block_sum<G::THREADS>(acc, red_s, a.partials + (long long)rank * kPartialStride);
     }
     const float sc = t == 0 ? sc1 : sc2;
@@ -344,9 +377,10 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
       else psi[x] = reg_update(psi[x], v[x], mk<float>(vr[x], vi[x]), a.half_dtau, a.dtau, a.dtau_lo, sc);
     }
   }
+  const float nan = __int_as_float(-1);
 #pragma unroll
-  for (int x = 0; x < N; ++x) a.psi[row + x] = psi[x];
-  if (!ok && a.err) atomicExch(a.err, 1);
+  for (int x = 0; x < N; ++x) a.psi[row + x] = ok ? psi[x] : mk<float>(nan, nan);
+  res_close(ok, a.err, bars);
 }
 
 template <int N, bool VREAL, bool SUMS>

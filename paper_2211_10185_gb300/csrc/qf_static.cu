@@ -147,6 +147,7 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
                  &r.a.dtau_lo);
     r.a.kinetic = kinetic;
     r.a.nsteps = 1;
+    r.a.spin = kResSpin;
     if (launch_fft_res_static(n, r, !v_complex, sums != nullptr, st) != cudaSuccess) return QF_ECUDA;
     return sums ? static_sums(partials, nbr, dsc, sums, st) : QF_OK;
   }

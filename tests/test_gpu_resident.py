@@ -106,3 +106,16 @@ def test_allocation_free_step_matches_resident_step(n, complex_v):
     # (one step of the same arithmetic in another instantiation, and the sums of its input)
     assert _rel(psi.cpu().numpy().astype(np.complex128), lat.get_wavefunction()) < 2e-6 * (1 + math.log2(n))
     assert abs(sums[0].item() - np.linalg.norm(psi0) ** 2) < 1e-6 * np.linalg.norm(psi0) ** 2
+
+
+def test_resident_steps_whose_waits_run_out_end_and_say_so():
+    """The self-test runs resident steps that give up at their first wait; the lattice steps on as if
+    it had not been called, and so does one that shares the GPU."""
+    a, v, psi0 = _inputs(32, False)
+    plain, probed = _gpu(32, a, v, psi0, O.FFT_REL), _gpu(32, a, v, psi0, O.FFT_REL)
+    for lat in (plain, probed):
+        lat.step_n(5, tol=0.0, check_every=4, snap_every=0)
+    assert probed.lib.qf_selftest_bounded_wait(probed.h) == Q.QF_ETIMEOUT
+    for lat in (plain, probed):
+        lat.step_n(6, tol=0.0, check_every=4, snap_every=0)
+    assert np.array_equal(plain.get_wavefunction(), probed.get_wavefunction())
