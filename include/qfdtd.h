@@ -386,9 +386,9 @@ const char* qf_batch_last_error(const qf_batch* b);
 const char* qf_last_error(const qf_lattice* lat);
 
 /* Self-test of the bounded device waits (no counterpart in the paper; failure
- * detection).  Launches, on the handle's stream, a kernel whose wait on a
- * shared-memory barrier can never complete; the wait gives up after its iteration limit
- * (about a second), the kernel records the failure and returns; then resident FFT steps of
+ * detection).  Launches, on the handle's stream, a kernel whose wait (the one that resident
+ * FFT steps use, with a short limit) is for bytes that nobody sends; the wait gives up,
+ * the kernel records the failure and returns; then resident FFT steps of
  * 8^3 sites in the handle's scratch field whose waits are given no time.  This call returns
  * QF_ETIMEOUT with the context still usable.  QF_OK would mean that a limit did not work. */
 qf_status qf_selftest_bounded_wait(qf_lattice* lat);

@@ -31,7 +31,6 @@ bool line_supported(int n);
 int line_final_blocks(int n);
 cudaError_t launch_fft2_group_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
 cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st);
-cudaError_t launch_bounded_wait_probe(int* err, cudaStream_t st);
 template <typename R>
 cudaError_t launch_stencil(const StencilGroup<R>& g, cudaStream_t st);
 template <typename R>
@@ -1445,7 +1444,7 @@ extern "C" qf_status qf_selftest_bounded_wait(qf_lattice* lat) {
   if (!lat) return QF_EINVAL;
   int* flag = &lat->sc()->err[1];
   QF_CUDA(lat, cudaMemsetAsync(flag, 0, sizeof(int), lat->st));
-  QF_CUDA(lat, launch_bounded_wait_probe(flag, lat->st));
+  QF_CUDA(lat, launch_bounded_wait_probe(flag, 1u << 16, lat->st));
   int err = 0;
   QF_CUDA(lat, cudaMemcpyAsync(&err, flag, sizeof(int), cudaMemcpyDeviceToHost, lat->st));
   QF_CUDA(lat, cudaStreamSynchronize(lat->st));

@@ -102,4 +102,19 @@ cudaError_t launch_fft_res_static(int n, const ResStatic& g, bool v_real, bool r
   }
 }
 
+__global__ void bounded_wait_probe(int* err, unsigned spin) {
+  __shared__ alignas(8) unsigned long long bar;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"((unsigned)__cvta_generic_to_shared(&bar)) : "memory");
+    res_expect(&bar, 16);  // no copy follows
+  }
+  __syncthreads();
+  const bool done = res_wait(&bar, 0, true, spin);
+  if (__syncthreads_or(done) == 0 && threadIdx.x == 0) atomicExch(err, 1);
+}
+cudaError_t launch_bounded_wait_probe(int* err, unsigned spin, cudaStream_t st) {
+  bounded_wait_probe<<<1, 32, 0, st>>>(err, spin);
+  return cudaGetLastError();
+}
+
 }  // namespace qf

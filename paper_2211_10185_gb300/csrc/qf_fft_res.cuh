@@ -399,6 +399,9 @@ __global__ void __launch_bounds__(ResG<N>::THREADS) fft_res_static_kernel(const 
 // with `reduce` one step and its check sums.
 cudaError_t launch_fft_res(int n, const ResGroup& g, bool v_real, bool reduce, cudaStream_t st);
 cudaError_t launch_fft_res_static(int n, const ResStatic& g, bool v_real, bool reduce, cudaStream_t st);
+// Self-test of res_wait: one block waits, `spin` tries, for bytes that nobody sends; *err is set when
+// every thread's wait ran out.
+cudaError_t launch_bounded_wait_probe(int* err, unsigned spin, cudaStream_t st);
 // Partial-sum rows of a member; 0 where the size has no resident form or the device cannot
 // run its cluster.
 int fft_res_blocks(int n);

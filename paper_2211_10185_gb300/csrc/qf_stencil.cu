@@ -59,25 +59,6 @@ cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Self-test of the bounded waits: an mbarrier that expects bytes nobody sends never
-// completes, so every thread's bounded wait runs out and the block reports it.
-__global__ void bounded_wait_probe(int* err) {
-  __shared__ alignas(8) unsigned long long bar;
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    mbar_expect_tx(&bar, 16);  // no copy follows
-  }
-  __syncthreads();
-  const bool ok = mbar_wait_bounded(&bar, 0);
-  if (__syncthreads_and(ok) == 0 && threadIdx.x == 0) atomicExch(err, 1);
-}
-
-cudaError_t launch_bounded_wait_probe(int* err, cudaStream_t st) {
-  bounded_wait_probe<<<1, 32, 0, st>>>(err);
-  return cudaGetLastError();
-}
-
 template cudaError_t launch_stencil<float>(const StencilGroup<float>&, cudaStream_t);
 template cudaError_t launch_stencil<double>(const StencilGroup<double>&, cudaStream_t);
 

@@ -119,3 +119,38 @@ def test_resident_steps_whose_waits_run_out_end_and_say_so():
     for lat in (plain, probed):
         lat.step_n(6, tol=0.0, check_every=4, snap_every=0)
     assert np.array_equal(plain.get_wavefunction(), probed.get_wavefunction())
+
+
+def _set_error_flag(lat):
+    """Sets the flag that a run-out wait sets: the last int pair but one double of the scalars, which
+    lie before the staging area at the workspace's end (256-byte multiples)."""
+    import torch
+
+    up = lambda x: (x + 255) // 256 * 256
+    total, scalars = lat.info()["workspace_bytes"], 32 * 8
+    at = total - up(min(16 * lat.n ** 3, 32 << 20)) - up(scalars) + scalars - 16
+    flag = lat.workspace[at:at + 8].view(torch.int32)
+    assert flag.tolist() == [0, 0]
+    torch.cuda.synchronize()
+    flag[0] = 1
+    torch.cuda.synchronize()
+    return flag
+
+
+def test_a_run_out_wait_is_reported_once_by_steps_and_batches():
+    from paper_2211_10185_gb300.serve import Batch
+
+    a, v, psi0 = _inputs(16, False)
+    lat = _gpu(16, a, v, psi0, O.FFT_REL)
+    flag = _set_error_flag(lat)
+    with pytest.raises(Q.QFError) as e:
+        lat.step_n(3, tol=0.0, check_every=0, snap_every=0)
+    assert e.value.status == Q.QF_ETIMEOUT and flag.tolist() == [0, 0]
+    lat.step_n(3, tol=0.0, check_every=0, snap_every=0)
+    b = Batch()
+    b.add(lat, 100, 0.0)
+    _set_error_flag(lat)
+    with pytest.raises(Q.QFError) as e:
+        b.step(3, check_every=0)
+    assert e.value.status == Q.QF_ETIMEOUT and flag.tolist() == [0, 0]
+    b.step(3, check_every=0)
