@@ -544,11 +544,22 @@ extern "C" qf_status qf_field_pointer(qf_lattice* lat, int slot, void** dev_ptr)
   return QF_OK;
 }
 
-// dtau of the update in the resident and plane forms (kinetic_dtau).
-static void form_dtau(const qf_lattice* lat, float tcoef, float* hi, float* lo) {
+// Coefficient of T(k) (FftPassArgs::tcoef) in double precision.
+static double exact_tcoef(const qf_lattice* lat) {
   const double n3 = (double)lat->d.n * lat->d.n * lat->d.n, a = lat->d.a;
-  const double exact = lat->kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * lat->mass * n3);
-  kinetic_dtau(lat->d.n, lat->dtau, exact, tcoef, hi, lo);
+  return lat->kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * lat->mass * n3);
+}
+// dtau of the update in the resident, plane and line forms (kinetic_dtau).
+static void form_dtau(const qf_lattice* lat, float tcoef, float* hi, float* lo) {
+  kinetic_dtau(lat->d.n, lat->dtau, exact_tcoef(lat), tcoef, hi, lo);
+}
+// Factor of the check sums of <psi|H_K psi>: kinetic_correction where one of those forms made them
+// (a step's; a field that is not stepped is measured by the plane form or by plain kernels).
+static double sums_correction(const qf_lattice* lat, bool step) {
+  const bool plane = uses_fft2(lat) && plane_supported(lat->d.n);
+  if (!plane && !(step && (uses_line(lat) || uses_res(lat)))) return 1.0;
+  const double t = exact_tcoef(lat);
+  return kinetic_correction(lat->d.n, t, (float)t);
 }
 
 template <typename R>
@@ -561,14 +572,12 @@ static const R* inv_of(const qf_lattice* lat) {
 // qf_stencil.cu); `in` is the field the kinetic term acts on.
 template <typename R>
 static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduce, const double* scale) {
-  const int n = lat->d.n;
   const double a = lat->d.a, m = lat->mass, dt = lat->dtau;
-  const double n3 = (double)n * n * n;
   FftPassArgs<R> p{};
   p.twiddle = reinterpret_cast<const cpx<R>*>(lat->ws + lat->L.tw);
   p.symbol = reinterpret_cast<const R*>(lat->ws + lat->L.sym);
   p.kinetic = lat->kinetic;
-  p.tcoef = (R)(lat->kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * m * n3));
+  p.tcoef = (R)exact_tcoef(lat);
   p.am2 = (R)((a * m) * (a * m));
   p.psi = reinterpret_cast<cpx<R>*>(in);
   p.v = lat->ws + lat->L.v;
@@ -861,7 +870,9 @@ static cudaError_t after_step(qf_lattice* lat, bool check, int nb, int snap_ever
   if (check) {
     const int interval = lat->renorm_step >= 0 ? (int)std::min<int64_t>(lat->step - lat->renorm_step, 1 << 30) : 0;
     cudaError_t e =
-        launch(lat, K_FINISH, [&] { return launch_finish(lat->partials(), nb, lat->sc(), 1, st, interval, lat->dtau); });
+        launch(lat, K_FINISH, [&] {
+          return launch_finish(lat->partials(), nb, lat->sc(), 1, st, interval, lat->dtau, sums_correction(lat, true));
+        });
     if (e != cudaSuccess) return e;
     lat->pending_scale = true;
     lat->K_check = k_in;
@@ -1120,7 +1131,9 @@ static qf_status measure(qf_lattice* lat, void* f, qf_energy* out) {
   int nb = 0;
   // FFT terms transform through tmp and read f; FDTD reads f only
   QF_CUDA(lat, kinetic_pass(lat, f, f, false, true, &lat->sc()->scale[0], &nb));
-  QF_CUDA(lat, launch(lat, K_FINISH, [&] { return launch_finish(lat->partials(), nb, lat->sc(), 0, lat->st); }));
+  QF_CUDA(lat, launch(lat, K_FINISH, [&] {
+    return launch_finish(lat->partials(), nb, lat->sc(), 0, lat->st, -1, 0.0, sums_correction(lat, false));
+  }));
   double e3[5];
   qf_status s = read_energy(lat, e3);
   if (s != QF_OK) return s;

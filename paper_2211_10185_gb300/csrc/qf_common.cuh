@@ -285,8 +285,9 @@ int stencil_blocks(int n);
 // energy; with set_scale also the step scales sc->scale[1..2] and their exponents k, j in
 // sc->energy[3..4].  interval > 0: steps since the field last had about unit norm, from
 // which the per-step decay is measured; interval 0: estimated from the energy and dtau.
+// kin multiplies the two sums of <psi|H_K psi>.
 cudaError_t launch_finish(const double* partials, int nblocks, DevScalars* sc, int set_scale,
-                          cudaStream_t st, int interval = -1, double dtau = 0.0);
+                          cudaStream_t st, int interval = -1, double dtau = 0.0, double kin = 1.0);
 
 // Gram-Schmidt and field helpers (FP64 accumulation).
 template <typename R>

@@ -76,9 +76,11 @@ __device__ __forceinline__ bool finish_rows(const double* __restrict__ partials,
 
 __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const double* __restrict__ partials, int nblocks,
                                                      DevScalars* sc, int set_scale, int interval,
-                                                     double dtau) {
+                                                     double dtau, double kin) {
   double tot[kNumSums];
   if (!finish_rows(partials, nblocks, tot)) return;
+  tot[1] *= kin;
+  tot[2] *= kin;
   if (threadIdx.x == 0) {
     const double nrm = tot[0];
     for (int i = 0; i < kNumSums; ++i) sc->sums[i] = tot[i];
@@ -135,8 +137,8 @@ static cudaError_t launch_cluster(void (*kern)(KArgs...), int c, cudaStream_t st
 }
 
 cudaError_t launch_finish(const double* partials, int nblocks, DevScalars* sc, int set_scale, cudaStream_t st,
-                          int interval, double dtau) {
-  return launch_cluster(finish_kernel, finish_cluster(nblocks), st, partials, nblocks, sc, set_scale, interval, dtau);
+                          int interval, double dtau, double kin) {
+  return launch_cluster(finish_kernel, finish_cluster(nblocks), st, partials, nblocks, sc, set_scale, interval, dtau, kin);
 }
 
 // ------------------------------------------------------------------------------------

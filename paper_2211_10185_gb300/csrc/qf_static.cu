@@ -103,8 +103,8 @@ const HostTables& host_tables(int n) {
   return n == 8 ? t8 : n == 12 ? t12 : n == 16 ? t16 : n == 24 ? t24 : t32;
 }
 
-qf_status static_sums(const double* partials, int nb, DevScalars* dsc, double* sums, cudaStream_t st) {
-  if (launch_finish(partials, nb, dsc, 0, st) != cudaSuccess) return QF_ECUDA;
+qf_status static_sums(const double* partials, int nb, DevScalars* dsc, double* sums, cudaStream_t st, double kin) {
+  if (launch_finish(partials, nb, dsc, 0, st, -1, 0.0, kin) != cudaSuccess) return QF_ECUDA;
   if (cudaMemcpyAsync(sums, dsc->sums, kNumSums * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return QF_ECUDA;
   return QF_OK;
@@ -127,7 +127,8 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
   char* base = static_cast<char*>(base_v);
 
   const double n3 = (double)n * n * n;
-  const float tcoef = (float)(kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3));
+  const double exact = kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3);
+  const float tcoef = (float)exact;
   const float am2 = (float)((a * mass) * (a * mass));
   DevScalars* dsc = reinterpret_cast<DevScalars*>(base + kStaticScOff);
   double* partials = reinterpret_cast<double*>(base + kStaticPartialsOff);
@@ -143,13 +144,12 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
     r.a.tcoef = tcoef;
     r.a.am2 = am2;
     r.a.half_dtau = (float)(0.5 * dtau);
-    kinetic_dtau(n, dtau, kinetic == QF_KIN_FFT_REL ? 1.0 / (a * n3) : 1.0 / (2.0 * a * a * mass * n3), tcoef, &r.a.dtau,
-                 &r.a.dtau_lo);
+    kinetic_dtau(n, dtau, exact, tcoef, &r.a.dtau, &r.a.dtau_lo);
     r.a.kinetic = kinetic;
     r.a.nsteps = 1;
     r.a.spin = kResSpin;
     if (launch_fft_res_static(n, r, !v_complex, sums != nullptr, st) != cudaSuccess) return QF_ECUDA;
-    return sums ? static_sums(partials, nbr, dsc, sums, st) : QF_OK;
+    return sums ? static_sums(partials, nbr, dsc, sums, st, kinetic_correction(n, exact, tcoef)) : QF_OK;
   }
 
   // tables of this call (the array holds the previous call's): per-stage twiddles, the
@@ -194,5 +194,5 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
   for (int pass = 0; pass < kFftPasses; ++pass)
     // (its twiddle scratch holds the first radix plan's table only)
     if (launch_fft_pass<float>(n, pass, p, tmp, st, &nb, false) != cudaSuccess) return QF_ECUDA;
-  return sums ? static_sums(partials, nb, dsc, sums, st) : QF_OK;
+  return sums ? static_sums(partials, nb, dsc, sums, st, 1.0) : QF_OK;
 }

@@ -2,7 +2,15 @@
 
 An energy E = <T> + <V> with |E| << <T> shows every relative error of <T> enlarged by <T>/|E|.
 N = 96 takes the four-pass form unless another is asked for: bit for bit.
+
+The resident and plane forms correct <T> for the rounding of T(k)'s single-precision coefficient
+and for their transforms' mean gain.  Case: psi = (-1)^x, an eigenstate of Eq. HK2's T with symbol
+4, on N = 2^m, where every transform, product and sum is exact in FP32; the mass is one
+whose coefficient rounds by more than 5e-8; V = -(1 - 1e-3) <T>.  What is left of the error is the
+mean gain where this mode has none: at most 3 x 0.76e-8 (N = 16), and FP64 rounding: 3e-8 <T>.
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -52,3 +60,49 @@ def test_n96_takes_the_four_pass_form_alone_and_in_a_batch(kind):
     for lat in (plain, member):
         assert np.array_equal(lat.get_wavefunction(), four.get_wavefunction())
         assert lat.energies() == four.energies()
+
+
+def _cancelling(n, a=0.25):
+    """mass, psi and V (single precision), <T> and the exact energy of the case above."""
+    for i in range(1000):
+        m = 1.0 + 0.001 * i
+        t = 1.0 / (2 * a * a * m * n ** 3)
+        if abs(float(np.float32(t)) / t - 1) > 5e-8:
+            break
+    psi = np.broadcast_to((-1.0) ** np.arange(n), (n, n, n)).astype(np.complex128)
+    kin = 4 / (2 * m * a * a)
+    v = float(np.float32(-kin * (1 - 1e-3)))
+    return a, m, psi, v, kin, kin + v
+
+
+@pytest.mark.parametrize("n", [16, 32, 64])
+def test_energy_of_cancelling_terms_alone_and_in_a_batch(n):
+    from paper_2211_10185_gb300.serve import Batch
+
+    a, m, psi, v, kin, e = _cancelling(n)
+    lats = [_lattice(n, a, O.FFT_SYMANZIK, m, np.full((n, n, n), v), psi) for _ in range(3)]
+    lats[0].step_n(2, tol=0.0, check_every=2, snap_every=0)
+    b = Batch()
+    for lat in lats[1:]:
+        b.add(lat, 2, 0.0)
+    b.step(2, check_every=2)
+    for lat in lats:
+        assert abs(lat.energies()["e"] - e) < 3e-8 * kin
+
+
+@pytest.mark.parametrize("n", [16, 32])
+def test_sums_of_the_allocation_free_step(n):
+    import torch
+
+    from paper_2211_10185_gb300 import qfdtd as Q
+
+    a, m, psi, v, kin, e = _cancelling(n)
+    p = torch.from_numpy(psi).to(torch.complex64).cuda()
+    vd = torch.full((n, n, n), v, dtype=torch.float32, device="cuda")
+    sums = torch.empty(5, dtype=torch.float64, device="cuda")
+    st = Q.load().qf_fft_step_static(n, a, O.FFT_SYMANZIK, m, 0.01, C.c_void_p(p.data_ptr()), C.c_void_p(vd.data_ptr()), 0, 1.0,
+                                     C.c_void_p(sums.data_ptr()), None)
+    assert st == Q.QF_OK
+    torch.cuda.synchronize()
+    s = sums.cpu().numpy()
+    assert abs((s[1] + s[3]) / s[0] - e) < 3e-8 * kin
