@@ -124,8 +124,9 @@ __device__ __forceinline__ void tb_rows(F&& f, std::integer_sequence<int, I...>)
 }
 
 // One site: c and its neighbours, potential (vx, vy), output scale sc; live: whether the site
-// may be nonzero (else the result is a zero times the numerator).  The same operations, in
-// the same order, as fdtd_update after lap_of(six_sum).
+// may be nonzero (else the result is zero, whatever V holds there: a dead site reads V at an
+// index 0, where a caller may have put an infinite wall).  The same operations, in the same order,
+// as fdtd_update after lap_of(six_sum).
 template <bool VREAL>
 __device__ __forceinline__ pk tb_site(pk c, pk xm, pk xp, pk ym, pk yp, pk zm, pk zp, float vx, float vy, float hd,
                                       pk kd2, pk m6, float sc, bool live) {
@@ -133,8 +134,9 @@ __device__ __forceinline__ pk tb_site(pk c, pk xm, pk xp, pk ym, pk yp, pk zm, p
   const pk lap = pk_fma(m6, c, nbs);
   const float dx = fma_rn<float>(hd, vx, 1.f), tx = add_rn<float>(2.f, -dx);
   if constexpr (VREAL) {
-    const float inv = live ? scaled_inverse<float>(sc, dx) : 0.f;
-    return pk_mul(pk_fma(kd2, lap, pk_mul(pk_make(tx, tx), c)), pk_make(inv, inv));
+    const float inv = scaled_inverse<float>(sc, dx);
+    const pk u = pk_mul(pk_fma(kd2, lap, pk_mul(pk_make(tx, tx), c)), pk_make(inv, inv));
+    return live ? u : 0ull;
   } else {
     // (2 - d) psi = (tx - i dy) psi, d = dx + i dy
     const float dy = mul_rn<float>(hd, vy);
@@ -142,17 +144,17 @@ __device__ __forceinline__ pk tb_site(pk c, pk xm, pk xp, pk ym, pk yp, pk zm, p
     const float ax = fma_rn<float>(tx, cc.x, mul_rn<float>(dy, cc.y));
     const float ay = fma_rn<float>(tx, cc.y, -mul_rn<float>(dy, cc.x));
     const cpx<float> nn = pk_get(pk_fma(kd2, lap, pk_make(ax, ay)));
-    const float inv = live ? scaled_inverse<float>(sc, fma_rn<float>(dx, dx, mul_rn<float>(dy, dy))) : 0.f;
-    return pk_make(mul_rn<float>(fma_rn<float>(nn.x, dx, mul_rn<float>(nn.y, dy)), inv),
-                   mul_rn<float>(fma_rn<float>(nn.y, dx, -mul_rn<float>(nn.x, dy)), inv));
+    const float inv = scaled_inverse<float>(sc, fma_rn<float>(dx, dx, mul_rn<float>(dy, dy)));
+    const pk u = pk_make(mul_rn<float>(fma_rn<float>(nn.x, dx, mul_rn<float>(nn.y, dy)), inv),
+                         mul_rn<float>(fma_rn<float>(nn.y, dx, -mul_rn<float>(nn.x, dy)), inv));
+    return live ? u : 0ull;
   }
 }
 
 // The two steps for output columns [28 bx, 28 bx + 28), rows [y0, y0 + 4) and planes [z0, z1)
 // of the lattice in g.  EDGE: some row of the warp's levels is row 0 or lies outside the
-// lattice.  Positions that must read as zero are redirected to plane 0 or column 0 (zero);
-// a dead position next to one that holds a non-finite value is zero in the output all the
-// same (selected), and its level-1 value only reaches positions that are non-finite already.
+// lattice.  Positions that must read as zero are redirected to plane 0 or column 0 (zero); dead
+// positions are zero at both levels by selection, whatever V or a neighbour holds.
 template <bool VREAL, bool EDGE, bool PRE>
 __device__ __forceinline__ void stencil_tb_march(const StencilTbArgs& g, int bx, int y0, int z0, int z1) {
   using u64 = unsigned long long;
@@ -225,11 +227,11 @@ __device__ __forceinline__ void stencil_tb_march(const StencilTbArgs& g, int bx,
         const pk c = B[K2][i + 1];
         const pk xm = __shfl_up_sync(0xffffffffu, c, 1), xp = __shfl_down_sync(0xffffffffu, c, 1);
         const pk u = tb_site<VREAL>(c, xm, xp, B[K2][i], B[K2][i + 2], B[K1][i + 1], B[K][i + 1], vx[K2][i + 1],
-                                    VREAL ? 0.f : vy[VREAL ? 0 : K2][VREAL ? 0 : i + 1], hd, kd2, m6, sc2, true);
-        const pk o = xlive && q >= 1 && ylive(y0 + i) ? u : 0ull;
+                                    VREAL ? 0.f : vy[VREAL ? 0 : K2][VREAL ? 0 : i + 1], hd, kd2, m6, sc2,
+                                    xlive && q >= 1 && ylive(y0 + i));
         const int st = xout && (!EDGE || y0 + i < n);
         asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %2, 0;\n @p st.global.b64 [%0], %1;\n}\n" ::"l"(
-                         tb_addr<i>(dst, s8)), "l"(o), "r"(st) : "memory");
+                         tb_addr<i>(dst, s8)), "l"(u), "r"(st) : "memory");
       }, std::make_integer_sequence<int, TB_ROWS>{});
     }
   };

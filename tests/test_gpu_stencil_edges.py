@@ -78,3 +78,20 @@ def test_complex_fp64_steps(n, complex_v):
     assert np.linalg.norm((got - ref).ravel()) < 1e-14 * 12 * np.linalg.norm(ref.ravel())
     assert abs(e - er) < 1e-12 * abs(er)
     assert not got[0].any() and not got[:, 0].any() and not got[:, :, 0].any()
+
+
+@pytest.mark.parametrize("wall", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("complex_v", [False, True])
+@pytest.mark.parametrize("n", [8, 30, 58, 200])
+def test_potential_on_the_dirichlet_planes_is_not_used(n, complex_v, wall):
+    """V there multiplies a psi that is zero: an infinite wall or no number changes no bit, in single
+    steps and in pairs.  (200: with the prefetch of the larger sizes.)"""
+    a, v, psi0 = _inputs(n, complex_v)
+    walled = v.copy()
+    w = complex(wall, wall) if complex_v else wall
+    walled[0], walled[:, 0], walled[:, :, 0] = w, w, w
+    want, e = _run(n, a, v, psi0, "c64", 1, 11)
+    assert np.isfinite(want).all()
+    for tblock in (1, 2):
+        got, eg = _run(n, a, walled, psi0, "c64", tblock, 11)
+        assert np.array_equal(got, want) and eg == e
