@@ -372,16 +372,16 @@ static qf_status staged_upload(qf_lattice* lat, const double* host, long long n,
   return QF_OK;
 }
 
-// The table of 1/(1 + dtau V/2) of complex-FP64 lattices with a real potential (behind it in its
-// field), and its renewal once both the potential and the time step are set.
-static double* inv_table(const qf_lattice* lat) {
+// The table of 1 - coef_A of complex-FP64 lattices with a real potential (behind it in its field), and
+// its renewal once both the potential and the time step are set.
+static double* coef_table(const qf_lattice* lat) {
   return !lat->c64() && lat->v_real ? reinterpret_cast<double*>(lat->ws + lat->L.v) + lat->sites : nullptr;
 }
-static cudaError_t renew_inv_table(qf_lattice* lat) {
-  double* inv = lat->have_v && lat->kinetic >= 0 ? inv_table(lat) : nullptr;
-  if (!inv) return cudaSuccess;
+static cudaError_t renew_coef_table(qf_lattice* lat) {
+  double* tab = lat->have_v && lat->kinetic >= 0 ? coef_table(lat) : nullptr;
+  if (!tab) return cudaSuccess;
   return launch(lat, K_CONVERT, [&] {
-    return launch_inverse_table(inv, reinterpret_cast<const double*>(lat->ws + lat->L.v), 0.5 * lat->dtau, lat->sites, lat->st);
+    return launch_coef_table(tab, reinterpret_cast<const double*>(lat->ws + lat->L.v), 0.5 * lat->dtau, lat->sites, lat->st);
   });
 }
 
@@ -419,7 +419,7 @@ extern "C" qf_status qf_set_potential(qf_lattice* lat, const double* v_re, const
   lat->v_real = (v_im == nullptr);
   drop_graphs(lat);
   lat->reset_plateau();
-  QF_CUDA(lat, renew_inv_table(lat));
+  QF_CUDA(lat, renew_coef_table(lat));
   return QF_OK;
 }
 
@@ -466,7 +466,7 @@ extern "C" qf_status qf_set_kinetic(qf_lattice* lat, int kinetic, double mass, d
     delete[] s;
     if (e != cudaSuccess) return cuda_fail(lat, e, "symbol upload");
   }
-  QF_CUDA(lat, renew_inv_table(lat));
+  QF_CUDA(lat, renew_coef_table(lat));
   return QF_OK;
 }
 
@@ -563,8 +563,8 @@ static double sums_correction(const qf_lattice* lat, bool step) {
 }
 
 template <typename R>
-static const R* inv_of(const qf_lattice* lat) {
-  if constexpr (sizeof(R) == 8) return inv_table(lat);
+static const R* coef_of(const qf_lattice* lat) {
+  if constexpr (sizeof(R) == 8) return coef_table(lat);
   else return nullptr;
 }
 
@@ -582,7 +582,7 @@ static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduc
   p.psi = reinterpret_cast<cpx<R>*>(in);
   p.v = lat->ws + lat->L.v;
   p.v_real = lat->v_real;
-  if constexpr (sizeof(R) == 8) p.inv = inv_table(lat);
+  if constexpr (sizeof(R) == 8) p.coef_u = coef_table(lat);
   p.half_dtau = (R)(0.5 * dt);
   p.dtau = (R)dt;
   p.scale = scale;
@@ -623,7 +623,7 @@ static StencilArgs<R> stencil_args(qf_lattice* lat, void* in, void* out, bool wr
                                    const double* scale) {
   const double a = lat->d.a, m = lat->mass, dt = lat->dtau;
   return StencilArgs<R>{reinterpret_cast<const cpx<R>*>(in), reinterpret_cast<cpx<R>*>(out), lat->ws + lat->L.v,
-                        lat->v_real, inv_of<R>(lat), (R)(1.0 / (2.0 * m * a * a)), (R)(0.5 * dt), (R)dt,
+                        lat->v_real, coef_of<R>(lat), (R)(1.0 / (2.0 * m * a * a)), (R)(0.5 * dt), (R)dt,
                         (R)(dt / (2.0 * m * a * a)), scale, lat->partials(),
                         write ? 1 : 0, reduce ? 1 : 0};
 }

@@ -77,7 +77,7 @@ struct FftPassArgs {
   cpx<R>* psi;            // psi_t in, psi_{t+1} out (same sites)
   const void* v;          // potential: cpx<R> (complex) or R (real)
   int v_real;
-  const R* inv;           // complex FP64 and real V: 1/(1 + dtau V/2) per site (else null)
+  const R* coef_u;        // complex FP64 and real V: 1 - coef_A per site (else null)
   R half_dtau;            // dtau / 2
   R dtau;
   R dtau_lo;              // second part of dtau in the plane form (else unused)
@@ -105,7 +105,7 @@ struct StencilArgs {
   cpx<R>* out;            // may be null when only measuring
   const void* v;
   int v_real;
-  const R* inv;           // as in FftPassArgs
+  const R* coef_u;        // as in FftPassArgs
   R kcoef;                // 1/(2 m a^2)
   R half_dtau;
   R dtau;
@@ -316,8 +316,8 @@ template <typename R>
 cudaError_t launch_real_from_f64(R* dst, const double* src, long long n, cudaStream_t st);
 template <typename R>
 cudaError_t launch_pack_f64(cpx<R>* dst, const double* re, const double* im, long long n, cudaStream_t st);
-// inv = 1/(1 + half_dtau v) per site
-cudaError_t launch_inverse_table(double* inv, const double* v, double half_dtau, long long n, cudaStream_t st);
+// u = 1 - coef_A = 2 w/(1 + w), w = half_dtau v, per site
+cudaError_t launch_coef_table(double* u, const double* v, double half_dtau, long long n, cudaStream_t st);
 int field_blocks();
 // Radial momentum histogram of a transformed field (shells b = round(|n|)); see
 // qf_fields.cu.  part: per-block integer histograms (blocks x nb); out: prob[nb].

@@ -424,10 +424,10 @@ __device__ __forceinline__ void fft_x_body(const FftPassArgs<R>& a, const int bi
           // division, a few ulp; FP64: correctly rounded)
           const cpx<R> vi = vat(i);
           if constexpr (VREAL && sizeof(R) == 8) {
-            // the reciprocal from the lattice's table: coef_A = 2/d - 1
-            const R is = a.inv[base + e_out<N, S - 1, PL>(g, b, r)] * sc;
-            const R ca = fma(R(2), is, -sc), cb = a.dtau * is;
-            v[i] = mk<R>(fma(ca, pv[i].x, -(cb * v[i].x)), fma(ca, pv[i].y, -(cb * v[i].y)));
+            // u = 1 - coef_A from the lattice's table: psi' = sc (psi - u psi - dtau (1 - u/2) H_K psi)
+            const R u = a.coef_u[base + e_out<N, S - 1, PL>(g, b, r)];
+            const R us = u * sc, cb = fma(-a.half_dtau, u, a.dtau) * sc;
+            v[i] = mk<R>(fma(sc, pv[i].x, -fma(us, pv[i].x, cb * v[i].x)), fma(sc, pv[i].y, -fma(us, pv[i].y, cb * v[i].y)));
           } else if constexpr (VREAL) {
             const R d = R(1) + a.half_dtau * vi.x;
             const cpx<R> num = cscale<R>(pv[i], R(2) - d) - cscale<R>(v[i], a.dtau);

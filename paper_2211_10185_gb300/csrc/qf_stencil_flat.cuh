@@ -71,7 +71,7 @@ __device__ __forceinline__ cpx<R> fdtd_update(cpx<R> c, cpx<R> lap, cpx<R> v, bo
 // lane is lost on sizes that 32 does not divide) and marches through zc planes with the
 // z-neighbours in registers; the four in-plane neighbours come through L1 and L2.  Nothing is
 // staged in shared memory.  What bounds it: the FP64 pipe in complex FP64 (2 fused
-// multiply-adds per clock and SM: 17 per site with the reciprocal table of a real V, 29
+// multiply-adds per clock and SM: 20 per site with the table of a real V, 29
 // without), HBM and L2 in complex FP32, latency on small lattices, which need as many blocks as
 // they have rows: the 32 x 32 tiles of 8 planes used before left all but 4 SMs idle at N = 32.
 // One step, before and now (in brackets: without the table): complex FP64 N = 32: 69 / 3.6 (4.5)
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kFlatThreads) stencil_flat_kernel(const __grid
   const bool hxm = live && x > 1, hxp = live && x + 1 < n, hym = live && y > 1, hyp = live && y + 1 < n;
   const cpx<R> zero = mk<R>(R(0), R(0));
   const cpx<R>* __restrict__ in = a.in;
-  const R sc = R(*a.scale), c26 = R(2) - R(6) * a.kd;
+  const R sc = R(*a.scale), ks = a.kd * sc, khs = R(0.5) * ks;
   CheckSums<R> cs;
   long long site = (long long)z0 * n2 + p;
   cpx<R> zm = zero, c = zero;
@@ -146,16 +146,17 @@ __global__ void __launch_bounds__(kFlatThreads) stencil_flat_kernel(const __grid
       if (hxp) xp = in[site + 1];
       if (hym) ym = in[site - n];
       if (hyp) yp = in[site + n];
-      if (live && (sizeof(R) == 4 || !a.inv || a.reduce)) vv = a.v_real ? mk<R>(reinterpret_cast<const R*>(a.v)[site], R(0)) : reinterpret_cast<const cpx<R>*>(a.v)[site];
+      if (live && (sizeof(R) == 4 || !a.coef_u || a.reduce)) vv = a.v_real ? mk<R>(reinterpret_cast<const R*>(a.v)[site], R(0)) : reinterpret_cast<const cpx<R>*>(a.v)[site];
     }
     if (live && up) {
       const cpx<R> nbs = six_sum<R>(xm, xp, ym, yp, zm, zp);
       if constexpr (sizeof(R) == 8) {
-        if (a.inv && a.write_psi && !a.reduce) {
-          // psi' = sc ((2 - 6 kd) / d - 1) psi + sc kd / d nbs: 17 FP64 operations a site, 1/d from
-          // the lattice's table, where lap, the update and the division take 29
-          const R is = a.inv[site] * sc, ca = fma(c26, is, -sc), cb = a.kd * is;
-          a.out[site] = mk<R>(fma(ca, c.x, cb * nbs.x), fma(ca, c.y, cb * nbs.y));
+        if (a.coef_u && a.write_psi && !a.reduce) {
+          // psi' = sc (psi - u psi + kd (1 - u/2) lap), u = 1 - coef_A from the lattice's table: 20
+          // FP64 operations a site, where lap, the update and the division take 29
+          const R u = a.coef_u[site], us = u * sc, cb = fma(-khs, u, ks);
+          const cpx<R> lap = lap_of<R>(c, nbs);
+          a.out[site] = mk<R>(fma(sc, c.x, -fma(us, c.x, -(cb * lap.x))), fma(sc, c.y, -fma(us, c.y, -(cb * lap.y))));
           zm = c;
           c = zp;
           continue;
