@@ -380,9 +380,11 @@ static double* coef_table(const qf_lattice* lat) {
 static cudaError_t renew_coef_table(qf_lattice* lat) {
   double* tab = lat->have_v && lat->kinetic >= 0 ? coef_table(lat) : nullptr;
   if (!tab) return cudaSuccess;
-  return launch(lat, K_CONVERT, [&] {
+  const cudaError_t e = launch(lat, K_CONVERT, [&] {
     return launch_coef_table(tab, reinterpret_cast<const double*>(lat->ws + lat->L.v), 0.5 * lat->dtau, lat->sites, lat->st);
   });
+  // complete on return, like every upload: a batch steps the lattice on another stream
+  return e == cudaSuccess ? cudaStreamSynchronize(lat->st) : e;
 }
 
 extern "C" qf_status qf_set_potential(qf_lattice* lat, const double* v_re, const double* v_im) {

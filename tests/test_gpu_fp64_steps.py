@@ -64,3 +64,23 @@ def test_many_fp64_steps_against_extended_precision(kind, n, a, seed, tol):
     ref = _extended(kind, n, a, 0.9, lat.info()["dtau"], v, psi)
     off = (lat.get_wavefunction().astype(np.clongdouble) - ref).ravel()
     assert float(np.sqrt((np.abs(off) ** 2).sum() / (np.abs(ref) ** 2).sum())) < tol
+
+
+def test_setting_potential_or_time_step_returns_with_its_work_done():
+    """A batch may step the lattice on another stream right after: nothing is left on the lattice's."""
+    import ctypes as C
+
+    from paper_2211_10185_gb300 import qfdtd as Q
+    from paper_2211_10185_gb300.lattice import Lattice
+
+    n = 160
+    lat = Lattice(n, 0.1, precision="c128")
+    v = np.ascontiguousarray(I.cornell(n, 0.1, 0.4, 0.2)).reshape(-1)
+    lat.set_kinetic(O.FDTD, 1.0)
+    lat.set_potential(v)
+    for _ in range(20):
+        assert lat.lib.qf_set_kinetic(lat.h, C.c_int(O.FDTD), C.c_double(1.0), C.c_double(0.001)) == Q.QF_OK
+        assert lat.stream.query()
+    for _ in range(3):
+        assert lat.lib.qf_set_potential(lat.h, Q.dptr(v), None) == Q.QF_OK
+        assert lat.stream.query()
