@@ -8,7 +8,14 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "qf_per_device.h"
+
 namespace qf {
+
+inline int current_device() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
 
 template <typename R>
 struct __align__(2 * sizeof(R)) cpx {

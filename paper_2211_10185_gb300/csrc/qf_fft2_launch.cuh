@@ -63,8 +63,8 @@ constexpr bool kF2Pdl = N == 256;
 template <int N>
 cudaError_t launch_fft2_pass_n(int pass, const FftGroup<float>& g, cudaStream_t st) {
   using G = F2G<N>;
-  static const bool attrs = f2_set_attrs<N>();
-  (void)attrs;
+  static PerDevice done;
+  done.ready(current_device(), f2_set_attrs<N>);
   if (g.count < 1 || g.count > kGroupMax) return cudaErrorInvalidValue;
   const dim3 grid_b(G::B_BLOCKS, g.count), grid_ac(G::AC_BLOCKS, g.count);
   const bool vreal = g.a[0].v_real != 0, sums = g.a[0].reduce != 0, write = g.a[0].write_psi != 0;

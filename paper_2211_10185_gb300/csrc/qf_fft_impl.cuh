@@ -626,8 +626,8 @@ static cudaError_t pass_n(int pass, FftPassArgs<R> a, cpx<R>* tmp, cudaStream_t 
   using G = Geom<R, N>;
   const int gx = N * N / G::LC, gs = (N / G::L) * (N / G::P);
   const size_t sx = smem_x<R, N>(), ss = smem_s<R, N>();
-  static bool attr_done = false;
-  if (!attr_done) {
+  static PerDevice done;
+  done.ready(current_device(), [&] {
     set_x_attrs<R, N, false>(sx);
     cudaFuncSetAttribute(fft_s_kernel<R, N, 1, OP_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_s_kernel<R, N, 2, OP_MID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
@@ -635,8 +635,8 @@ static cudaError_t pass_n(int pass, FftPassArgs<R> a, cpx<R>* tmp, cudaStream_t 
     cudaFuncSetAttribute(fft_s_kernel<R, N, 2, OP_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_s_kernel<R, N, 2, OP_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_x_kernel<R, N, OP_INV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sx);
-    attr_done = true;
-  }
+    return true;
+  });
   if (nfinal) *nfinal = gx;
   FftPassArgs<R> p = a;
   p.data = tmp;
@@ -666,8 +666,8 @@ template <typename R, int N, int V = 0>
 static cudaError_t group_pass_n(int pass, const FftGroup<R>& g, cudaStream_t st) {
   using G = Geom<R, N, V>;
   const size_t sx = smem_x<R, N, V>(), ss = smem_s<R, N, V>();
-  static bool attr_done = false;
-  if (!attr_done) {
+  static PerDevice done;
+  done.ready(current_device(), [&] {
     set_x_attrs<R, N, true, V>(sx);
     cudaFuncSetAttribute(fft_s_group_kernel<R, N, 1, OP_FWD, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_s_group_kernel<R, N, 2, OP_MID, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
@@ -675,8 +675,8 @@ static cudaError_t group_pass_n(int pass, const FftGroup<R>& g, cudaStream_t st)
     cudaFuncSetAttribute(fft_s_group_kernel<R, N, 2, OP_FWD, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_s_group_kernel<R, N, 2, OP_INV, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
     cudaFuncSetAttribute(fft_x_group_kernel<R, N, OP_INV, false, false, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sx);
-    attr_done = true;
-  }
+    return true;
+  });
   const dim3 gx(N * N / G::LC, g.count), gs((N / G::L) * (N / G::P), g.count);
   const bool vreal = g.a[0].v_real != 0, sums = g.a[0].reduce != 0, write = g.a[0].write_psi != 0;
   const bool next = write && g.a[0].emit_next != 0;

@@ -18,8 +18,8 @@ static bool line_setup() {
 template <int N>
 static cudaError_t line_pass(int pass, const FftGroup<float>& g, cudaStream_t st) {
   using L = LineG<N>;
-  static const bool ready = line_setup<N>();
-  (void)ready;
+  static PerDevice done;
+  done.ready(current_device(), line_setup<N>);
   const dim3 gz(L::Z_BLOCKS, g.count), gx(L::X_BLOCKS, g.count);
   constexpr int tx = 32 * L::X_WARPS;
   if (pass == 2) {

@@ -36,8 +36,8 @@ static bool plane_setup() {
 template <int N>
 static cudaError_t plane_pass(int pass, const FftGroup<float>& g, cudaStream_t st) {
   using G = PlaneG<N>;
-  static const bool ready = plane_setup<N>();
-  (void)ready;
+  static PerDevice done;
+  done.ready(current_device(), plane_setup<N>);
   if (g.count < 1 || g.count > kGroupMax) return cudaErrorInvalidValue;
   const dim3 gp(N, g.count), gz(G::Z_BLOCKS, g.count);
   constexpr int tp = G::P_THREADS, tz = 32 * G::Z_WARPS;

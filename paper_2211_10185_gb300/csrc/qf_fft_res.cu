@@ -49,13 +49,13 @@ static bool res_setup() {
     int clusters = 0;
     ok = ok && cudaOccupancyMaxActiveClusters(&clusters, f, &cfg) == cudaSuccess && clusters > 0;
   }
-  cudaGetLastError();  // (a refusal above is an answer, not an error)
+  if (!ok) cudaGetLastError();  // (a refusal above is an answer, not an error)
   return ok;
 }
 template <int N>
 static bool res_ready() {
-  static const bool ok = res_setup<N>();
-  return ok;
+  static PerDevice done;
+  return done.ready(current_device(), res_setup<N>);
 }
 
 #define QF_RES_CASES QF_CASE(8) QF_CASE(12) QF_CASE(16) QF_CASE(24) QF_CASE(32)
