@@ -21,8 +21,7 @@
 //
 // What bounds it: the latency of a block's four transforms with 6-12 warps per SM, on N of the 152
 // SMs in P (the four-pass form: that of four launches, 11.6-25 us a step).  One step with
-// Eq. HK2, before and now: N = 48: 12.8 / 5.5 us, 64: 11.6-13 / 7.8, 96: 25.1 / 17.9; with
-// psi and V read behind the dependency instead of ahead of it 6.0, 9.0, 19.1.  N = 128 took 40 us
+// Eq. HK2, before and now: N = 48: 12.8 / 5.5 us, 64: 11.6-13 / 7.8, 96: 25.1 / 17.9 (not the default there).  N = 128 took 40 us
 // so (32 elements a thread, one block of 16 warps per SM, spills) against 25.7 in the split form.
 #pragma once
 #include "qf_fft_reg.cuh"
@@ -105,6 +104,14 @@ __device__ __forceinline__ int plane_idx(int y, int x) {
 __device__ __forceinline__ void plane_dependency() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+__device__ __forceinline__ cpx<float> plane_ld_early(const cpx<float>* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  cpx<float> c;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(w));
+  return c;
 }
 
 // Forward half: x lines in v -> plane, y forward, S.
@@ -221,18 +228,25 @@ __global__ void __launch_bounds__(PlaneG<N>::P_THREADS) plane_p_kernel(const __g
   const int xg = lane & 3, line = warp * 8 + (lane >> 2), cg = lane >> 3, col = warp * 8 + (lane & 7);
   const long long row = ((long long)z * N + line) * N + xg;
   plane_twiddles<N>(tw_s, G::P_THREADS);
-  // psi and V of the thread's sites x = xg + 4 m of its line: not written by the Z pass that this
-  // block may overlap, and everything before that pass is complete (it waited for it before
-  // it let this launch start), so they are read ahead of the dependency
+  // psi and V of the thread's sites x = xg + 4 m of its line, and the scale, are read ahead of the
+  // dependency (behind it a step takes 6.3 us instead of 5.8 at N = 48, 9.3 instead of 8.5 at 64).  The
+  // Z pass that this block may overlap writes none of them.  V is constant.  What wrote psi and
+  // the scale (P of the step before, the check's finishing sums) came before that Z pass, whose
+  // blocks let this launch start only behind their own griddepcontrol.wait, that is with those
+  // kernels complete and their writes performed in global memory.  This grid has not waited for
+  // them itself, so nothing promises that a first-level cache holds no older copy: these
+  // loads are relaxed at GPU scope, which L2 serves.
   cpx<float> psi[E], vv[VREAL ? 1 : E];
   float vr[VREAL ? E : 1];
 #pragma unroll
   for (int m = 0; m < E; ++m) {
-    psi[m] = a.psi[row + 4 * m];
+    psi[m] = plane_ld_early(a.psi + row + 4 * m);
     if constexpr (VREAL) vr[m] = reinterpret_cast<const float*>(a.v)[row + 4 * m];
     else vv[m] = reinterpret_cast<const cpx<float>*>(a.v)[row + 4 * m];
   }
-  const float sc = float(*a.scale);
+  double scale;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(scale) : "l"(a.scale) : "memory");
+  const float sc = float(scale);
   plane_dependency();
   cpx<float>* __restrict__ S = a.data;
   cpx<float> v[E];
