@@ -206,6 +206,9 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = *y_at(cg + 4 * m);
     plane_line<N, false>(v, cg, tw_s, y_at);
+    // a block of the cluster receives from two of the four lanes of a line only, and may store into
+    // this buffer once it has: no lane sends before all have read
+    __syncwarp();
     if (ok) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
@@ -223,6 +226,7 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
     for (int m = 0; m < E; ++m)
       v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[cg + 4 * m], a.tcoef, a.am2));
     plane_line<N, true>(v, cg, tw_s, z_at);
+    __syncwarp();  // (as above)
     if (ok) {
 #pragma unroll
       for (int m = 0; m < E; ++m) {
