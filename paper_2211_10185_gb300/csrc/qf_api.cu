@@ -553,7 +553,7 @@ static double exact_tcoef(const qf_lattice* lat) {
 }
 // dtau of the update in the resident, plane and line forms (kinetic_dtau).
 static void form_dtau(const qf_lattice* lat, float tcoef, float* hi, float* lo) {
-  kinetic_dtau(lat->d.n, lat->dtau, exact_tcoef(lat), tcoef, hi, lo);
+  kinetic_dtau(lat->d.n, fft_tile_variant(lat->d.n) >> 1, lat->dtau, exact_tcoef(lat), tcoef, hi, lo);
 }
 // Factor of the check sums of <psi|H_K psi>: kinetic_correction where one of those forms made them
 // (a step's; a field that is not stepped is measured by the plane form or by plain kernels).
@@ -561,7 +561,7 @@ static double sums_correction(const qf_lattice* lat, bool step) {
   const bool plane = uses_fft2(lat) && plane_supported(lat->d.n);
   if (!plane && !(step && (uses_line(lat) || uses_res(lat)))) return 1.0;
   const double t = exact_tcoef(lat);
-  return kinetic_correction(lat->d.n, t, (float)t);
+  return kinetic_correction(lat->d.n, fft_tile_variant(lat->d.n) >> 1, t, (float)t);
 }
 
 template <typename R>

@@ -144,12 +144,12 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
     r.a.tcoef = tcoef;
     r.a.am2 = am2;
     r.a.half_dtau = (float)(0.5 * dtau);
-    kinetic_dtau(n, dtau, exact, tcoef, &r.a.dtau, &r.a.dtau_lo);
+    kinetic_dtau(n, 0, dtau, exact, tcoef, &r.a.dtau, &r.a.dtau_lo);
     r.a.kinetic = kinetic;
     r.a.nsteps = 1;
     r.a.spin = kResSpin;
     if (launch_fft_res_static(n, r, !v_complex, sums != nullptr, st) != cudaSuccess) return QF_ECUDA;
-    return sums ? static_sums(partials, nbr, dsc, sums, st, kinetic_correction(n, exact, tcoef)) : QF_OK;
+    return sums ? static_sums(partials, nbr, dsc, sums, st, kinetic_correction(n, 0, exact, tcoef)) : QF_OK;
   }
 
   // tables of this call (the array holds the previous call's): per-stage twiddles, the
