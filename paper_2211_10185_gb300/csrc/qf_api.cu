@@ -28,6 +28,7 @@ int fft2_final_blocks(int n);
 int fft2_measure_blocks(int n);
 bool plane_supported(int n);
 bool line_supported(int n);
+bool line_has_pass(int n, int pass);
 int line_final_blocks(int n);
 cudaError_t launch_fft2_group_pass(int n, int pass, const FftGroup<float>& g, cudaStream_t st);
 cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st);
@@ -649,7 +650,9 @@ static std::mutex g_tune_mu;  // the autotuners' tables
 // On the first four-pass FFT step of a size, every variant (two tile geometries, times two
 // radix plans where the size has a second one) times the five passes of a step (the
 // reducing pass measuring only: psi is untouched, the scratch field is overwritten) and
-// the fastest is kept for the process.  Never runs while the stream is being captured.
+// the fastest is kept for the process.  A lattice that runs some passes in the line form times
+// the passes of its further steps that it leaves to these kernels.  Never runs while the stream
+// is being captured.
 static void tune_fft_tiles(qf_lattice* lat) {
   const int n = lat->d.n;
   if (!lat->c64() || lat->kinetic == QF_KIN_FDTD || uses_fft2(lat) || fft_tile_choice(n) >= 0) return;
@@ -668,12 +671,17 @@ static void tune_fft_tiles(qf_lattice* lat) {
   float best_ms = 1e30f;
   int best = 0;
   const int nvar = fft_has_alt_plan(n) ? 4 : 2;
+  std::vector<int> passes;
+  for (int ps = 0; ps < kFftPasses; ++ps)
+    if (!uses_line(lat) || (ps > 0 && !line_has_pass(n, ps))) passes.push_back(ps);
+  launch_fft_pass<float>(n, 0, p, p.data, lat->st, nullptr);  // (the scratch field may hold anything)
+  lat->launches += 1;
   for (int v = 0; v < nvar; ++v) {
     set_fft_tile_choice(n, v);
     auto step = [&] {
       cudaError_t e = cudaSuccess;
-      for (int ps = 0; ps < kFftPasses && e == cudaSuccess; ++ps)
-        e = launch_fft_pass<float>(n, ps, p, p.data, lat->st, nullptr);
+      for (size_t i = 0; i < passes.size() && e == cudaSuccess; ++i)
+        e = launch_fft_pass<float>(n, passes[i], p, p.data, lat->st, nullptr);
       return e;
     };
     bool ok = step() == cudaSuccess;  // warm-up
@@ -684,7 +692,7 @@ static void tune_fft_tiles(qf_lattice* lat) {
            cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
       tot += ms;
     }
-    lat->launches += 4 * kFftPasses;
+    lat->launches += 4 * (int64_t)passes.size();
     if (ok && tot < best_ms) {
       best_ms = tot;
       best = v;

@@ -61,3 +61,26 @@ def test_line_passes_match_four_pass_kernels(n, kind, complex_v):
         ref.step_n(steps, check_every=2, snap_every=0)
         assert _rel(got[True], ref.psi) < tol
         assert abs(e[True] - ref.energies()["e"]) < 1e-5 * abs(e[True])
+
+
+def test_autotuner_times_the_passes_that_the_line_form_leaves():
+    """One warm pass, then four rounds of two tile variants of the y passes (1 and 3) at N = 192, whose x
+    and z passes run in the line form: 17 launches before the first step's five."""
+    import ctypes as C
+
+    from paper_2211_10185_gb300 import qfdtd as Q
+    from paper_2211_10185_gb300.lattice import Lattice
+
+    n, lib, old = 192, Q.load(), C.c_int()
+    assert lib.qf_get_fft_tiles(n, C.byref(old)) == Q.QF_OK
+    try:
+        assert lib.qf_set_fft_tiles(n, -1) == Q.QF_OK
+        lat = Lattice(n, 0.1, precision="c64")
+        lat.set_potential(I.cornell(n, 0.1, 0.4, 0.2))
+        lat.set_kinetic(O.FFT_REL, 1.0)
+        lat.set_wavefunction(I.gaussian_field(n, 1))
+        before = lat.info()["launches"]
+        lat.step_n(1, tol=0.0, check_every=0, snap_every=0)
+        assert lat.info()["launches"] - before == 1 + 4 * 2 * 2 + 5
+    finally:
+        lib.qf_set_fft_tiles(n, old.value)
