@@ -157,6 +157,7 @@ struct qf_lattice {
     int64_t launches;  // kernels in the graph
   };
   std::vector<Graph> graphs;
+  uint64_t graph_gen = 0;  // counts what outdates captured steps of this lattice, a batch's too
   bool use_graphs = true;
   // FDTD steps fused per pass (1 or 2) and whether the live field is known to be zero on
   // the Dirichlet planes (it is after any FDTD step), which the two-step kernel needs
@@ -222,6 +223,7 @@ static bool default_form(int n) { return n != 96; }
 static void drop_graphs(qf_lattice* lat) {
   for (auto& g : lat->graphs) cudaGraphExecDestroy(g.exec);
   lat->graphs.clear();
+  lat->graph_gen += 1;
 }
 
 static qf_status fail(qf_lattice* lat, qf_status s, const std::string& msg) {
@@ -1717,7 +1719,8 @@ static qf_status batch_issue_step(qf_batch* b, const std::vector<int>& run, cons
 // The check_every - 1 steps after a check that every running member took together
 // issue the same launches each time the batch holds the same members in the same buffer
 // state, so they are captured once into a CUDA graph (keyed by members, FDTD buffer
-// parity, first-pass state and FDTD pairing) and replayed; the host bookkeeping of those
+// parity, first-pass state, FDTD pairing and the count of what else changes a member's launches,
+// such as the form of its FFT step) and replayed; the host bookkeeping of those
 // steps follows the replay.  FDTD members that qualify (pairable) take the interval's
 // steps two per launch from its first step on, the last one alone when the count is odd,
 // as a lone lattice does.  Returns QF_OK with *used = false when the interval does not
@@ -1737,8 +1740,8 @@ static qf_status batch_chunk_graph(qf_batch* b, const std::vector<int>& run, int
     if (!L->pending_scale || L->prof || L->step % check_every != 1 || mb.steps_done + k > mb.max_steps)
       return QF_OK;
     key.push_back(reinterpret_cast<uintptr_t>(L));
-    key.push_back((uintptr_t)((L->live & 1) | (L->xfwd_valid ? 2 : 0) | (uses_fft2(L) ? 4 : 0) |
-                              (pairable(L) ? 8 : 0) | (uses_res(L) ? 16 : 0)));
+    key.push_back((uintptr_t)((L->live & 1) | (L->xfwd_valid ? 2 : 0) | (pairable(L) ? 4 : 0)));
+    key.push_back((uintptr_t)L->graph_gen);
   }
   std::vector<char> pair(run.size(), 0);
   for (size_t q = 0; q < run.size(); ++q) {

@@ -84,3 +84,36 @@ def test_autotuner_times_the_passes_that_the_line_form_leaves():
         assert lat.info()["launches"] - before == 1 + 4 * 2 * 2 + 5
     finally:
         lib.qf_set_fft_tiles(n, old.value)
+
+
+def test_two_members_and_a_change_of_form_between_batch_steps():
+    """N = 192 with Eq. HK2, two members a launch, the form switched off and on again between intervals
+    that the batch replays from graphs: bit for bit what the lattices do alone."""
+    from paper_2211_10185_gb300.lattice import Lattice
+    from paper_2211_10185_gb300.serve import Batch
+
+    n, a = 192, 1.0 / 12
+
+    def pair():
+        out = []
+        for seed in (1, 2):
+            lat = Lattice(n, a, precision="c64", n_snap=1)
+            lat.set_potential(I.cornell(n, a, 0.3 + 0.1 * seed, 0.2))
+            lat.set_kinetic(O.FFT_SYMANZIK, 0.8 + 0.1 * seed)
+            lat.set_wavefunction(I.gaussian_field(n, seed))
+            out.append(lat)
+        return out
+
+    alone, members = pair(), pair()
+    b = Batch()
+    for lat in members:
+        b.add(lat, 1000, 0.0)
+    for line in (True, False, True):
+        for lat in alone + members:
+            lat.use_two_pass_fft(line)
+        b.step(16, check_every=8)
+        for lat, mem in zip(alone, members):
+            lat.step_n(16, tol=0.0, check_every=8, snap_every=8)
+            assert np.array_equal(mem.get_wavefunction(), lat.get_wavefunction()), line
+            assert mem.energies() == lat.energies()
+    assert b.graph_info()[1] >= 5
