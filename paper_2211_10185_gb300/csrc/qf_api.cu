@@ -766,8 +766,9 @@ static cudaError_t res_steps(qf_lattice* lat, int nsteps, bool reduce, const dou
 // How many steps of a resident lattice one launch takes from step t on: up to the next check,
 // the next snapshot or `left`, and no more than a launch of some milliseconds.  t is not a
 // check step.
+constexpr int64_t kResRunMax = 2048;
 static int64_t res_run(int64_t t, int64_t left, int check_every, int snap_every) {
-  int64_t k = std::min<int64_t>(left, 2048);
+  int64_t k = std::min(left, kResRunMax);
   if (check_every > 0) k = std::min<int64_t>(k, check_every - t % check_every);
   if (snap_every > 0) k = std::min<int64_t>(k, snap_every - t % snap_every);
   return k;
@@ -1770,8 +1771,11 @@ static qf_status batch_chunk_graph(qf_batch* b, const std::vector<int>& run, int
     QF_BCUDA(b, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     qf_status s = QF_OK;
     for (int j = 0; j < k && s == QF_OK; ++j) {
-      for (size_t q = 0; q < run.size(); ++q)
-        ns[q] = pair[q] ? ((j & 1) ? 0 : (j + 1 < k) ? 2 : 1) : uses_res(b->m[run[q]].lat) ? (j == 0 ? k : 0) : 1;
+      for (size_t q = 0; q < run.size(); ++q) {
+        if (pair[q]) ns[q] = (j & 1) ? 0 : (j + 1 < k) ? 2 : 1;
+        else if (uses_res(b->m[run[q]].lat)) ns[q] = j % kResRunMax == 0 ? (int)std::min<int64_t>(k - j, kResRunMax) : 0;
+        else ns[q] = 1;
+      }
       s = batch_issue_step(b, run, nochk, nblk, st, ns);
       for (size_t q = 0; q < run.size(); ++q) {
         qf_lattice* L = b->m[run[q]].lat;

@@ -154,3 +154,23 @@ def test_a_run_out_wait_is_reported_once_by_steps_and_batches():
         b.step(3, check_every=0)
     assert e.value.status == Q.QF_ETIMEOUT and flag.tolist() == [0, 0]
     b.step(3, check_every=0)
+
+
+def test_a_batch_cuts_long_intervals_like_a_lattice_alone():
+    """Intervals of 2100 steps: a launch takes 2048 at most, replayed from a graph too (per interval the
+    check step, its finishing sums and two launches)."""
+    from paper_2211_10185_gb300.serve import Batch
+
+    a, v, psi0 = _inputs(8, False)
+    alone, member = _gpu(8, a, v, psi0, O.FFT_SYMANZIK), _gpu(8, a, v, psi0, O.FFT_SYMANZIK)
+    for lat in (alone, member):
+        lat.set_kinetic(O.FFT_SYMANZIK, 0.9, 1e-3)  # (an interval decays by less than exp(-30))
+    alone.step_n(4200, tol=0.0, check_every=2100, snap_every=0)
+    b = Batch()
+    b.add(member, 10000, 0.0)
+    b.step(4200, check_every=2100, snap_every=0)
+    assert np.isfinite(alone.get_wavefunction()).all()
+    assert np.array_equal(alone.get_wavefunction(), member.get_wavefunction())
+    n = C.c_int64()
+    assert b.lib.qf_batch_info(b.h, C.byref(n)) == Q.QF_OK
+    assert b.graph_info()[1] == 2 and n.value == 2 * 4
