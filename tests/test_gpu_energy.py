@@ -106,3 +106,16 @@ def test_sums_of_the_allocation_free_step(n):
     torch.cuda.synchronize()
     s = sums.cpu().numpy()
     assert abs((s[1] + s[3]) / s[0] - e) < 3e-8 * kin
+
+
+@pytest.mark.parametrize("n", [16, 32, 48, 192])
+def test_a_mass_beyond_single_precision_leaves_the_potential_alone(n):
+    """1/(2 a^2 m N^3) is zero in FP32 for m = 1e45: every site decays by its own V.  Three steps of about
+    four roundings: 2e-6 as for one FFT step."""
+    a, dtau = 0.25, 0.01
+    v, psi = I.cornell(n, a, 0.45, 0.2), I.gaussian_field(n, 3)
+    lat = _lattice(n, a, O.FFT_SYMANZIK, 1.0, v, psi)
+    lat.set_kinetic(O.FFT_SYMANZIK, 1e45, dtau)
+    lat.step_n(3, tol=0.0, check_every=0, snap_every=0)
+    want = psi * ((1 - dtau * v / 2) / (1 + dtau * v / 2)) ** 3
+    assert np.linalg.norm((lat.get_wavefunction() - want).ravel()) < 2e-6 * np.linalg.norm(want.ravel())
