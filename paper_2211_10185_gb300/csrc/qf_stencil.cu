@@ -45,7 +45,7 @@ cudaError_t launch_stencil_tb(const StencilTbGroup& g, cudaStream_t st) {
   if (total > (1LL << 30)) return cudaErrorInvalidValue;
   gl.start[g.count] = (int)total;
   // the L2 prefetch pays for its instructions only where psi and V do not stay in L2 (N = 192:
-  // 43.5 / 43.4 us without / with it, N = 384: 280 / 259, N = 128: 18.3 / 18.9)
+  // 44.5 / 43.3 us without / with it, N = 250: 89.0 / 86.8, N = 384: 291 / 274, N = 128: 16.9 / 17.0)
   bool pre = true;
   for (int i = 0; i < g.count; ++i) pre = pre && g.m[i].n >= 192;
   const unsigned nb = (unsigned)total;

@@ -74,9 +74,9 @@ __device__ __forceinline__ cpx<R> fdtd_update(cpx<R> c, cpx<R> lap, cpx<R> v, bo
 // multiply-adds per clock and SM: 20 per site with the table of a real V, 29
 // without), HBM and L2 in complex FP32, latency on small lattices, which need as many blocks as
 // they have rows: the 32 x 32 tiles of 8 planes used before left all but 4 SMs idle at N = 32.
-// One step, before and now (in brackets: without the table): complex FP64 N = 32: 69 / 3.6 (4.5)
-// us, 64: 71 / 12 (16), 128: 133 / 88 (117); complex FP32 N = 32: 23 / 10 us, 250: 112 / 109,
-// 512: 783 / 786 (bracketed by events).
+// One step, tiles / now (mean of a run of steps): complex FP64 with real V N = 32: 69 / 4.3 us,
+// 64: 71 / 15, 128: 133 / 97, 160: 260 / 196; with complex V 64: 97 / 26, 128: 175 / 156, 160: 339 /
+// 295; complex FP32 N = 32: 23 / 4.2 us, 250: 112 / 76, 512: 783 / 559.
 constexpr int kFlatThreads = 128;
 
 // Members of one launch may have different lattice sizes: member i runs

@@ -14,12 +14,12 @@
 // rows meet in L1, came out 15-35 % slower).  The arithmetic is on packed pairs (re, im), one
 // instruction where two were needed, and the lane's address of a row is one instruction.
 //
-// What bounds it: instruction issue and load latency about equally (N = 256: 61 M warp
-// instructions, 56 % of issue slots, 16 warps per SM at 128 registers), not yet HBM (20
+// What bounds it: instruction issue and load latency about equally (N = 256: 68 M warp
+// instructions, 62 % of issue slots, 16 warps per SM at 128 registers), not yet HBM (20
 // bytes per site and two steps).  The form before kept both levels in shared memory
 // (TMA-filled 36 x 36 planes, seven reads a site, a block barrier per plane, about 190
-// instructions a site).  Two steps, before and now: N = 64: 31 / 10 us, 128: 25 / 18 us,
-// 250: 131 / 83 us (3.7 TB/s of the 20 bytes), 256: 134 / 95 us, 384: 402 / 259 us.
+// instructions a site).  Two steps, before and now: N = 64: 31 / 8.4 us, 128: 25 / 17 us,
+// 250: 131 / 86 us (3.6 TB/s of the 20 bytes), 256: 134 / 97 us, 384: 402 / 274 us.
 //
 // Sites with an index 0 (the Dirichlet planes) and sites outside the lattice are zero at
 // every level; the input field must already be zero on the Dirichlet planes (true after
@@ -71,9 +71,10 @@ __host__ __device__ inline int stencil_tb_member_blocks(int n, int nzb) {
 // resident warps per SM at 128 registers): a small lattice is bound by the latency of a
 // warp's march.  Beyond that as many chunks as make whole waves of resident warps, with at
 // least 16 planes each (a chunk repeats two planes of level 1 and four loads); one wave if
-// its chunks are shorter than that.  Measured, us per pass: N = 64: 12 (2-4 planes), 28 (16);
-// N = 192: 67 in one wave, 84 in 1.1; N = 250: 135 / 135 / 132 / 136 in 1 / 2 / 3 / 4 waves;
-// N = 384: 440 (3 waves), 401 (13), 430 (26).
+// its chunks are shorter than that.  Measured, us per pass: N = 64: 8.6 in chunks of 2 planes, 9.3 of
+// 4, 17 of 16; N = 192: 43.9 in one wave, 47.7 in 1.7; N = 250: 85.7 / 86.5 / 87.6 / 89.2 in
+// 1 / 2 / 3 / 4 waves, 96 in 7; N = 384: 315 in 1.7 waves, 281 in 2.8, 268 in 8, 275 in 13 (taken),
+// 297 in 26.
 inline int stencil_tb_chunks(int n) {
   const long long cap = 152 * 16, tiles = stencil_tb_member_blocks(n, 1);
   if (tiles * ((n + 1) / 2) <= cap) return (n + 1) / 2;
