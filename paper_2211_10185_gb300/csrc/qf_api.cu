@@ -558,6 +558,10 @@ static double exact_tcoef(const qf_lattice* lat) {
 static void form_dtau(const qf_lattice* lat, float tcoef, float* hi, float* lo) {
   kinetic_dtau(lat->d.n, fft_tile_variant(lat->d.n) >> 1, lat->dtau, exact_tcoef(lat), tcoef, hi, lo);
 }
+// Rest mass of Eq. HK3 in those forms (kinetic_rest).
+static void form_rest(const qf_lattice* lat, float tcoef, float* t0, float* t0_lo) {
+  kinetic_rest(lat->d.n, fft_tile_variant(lat->d.n) >> 1, lat->mass, exact_tcoef(lat), tcoef, t0, t0_lo);
+}
 // Factor of the check sums of <psi|H_K psi>: kinetic_correction where one of those forms made them
 // (a step's; a field that is not stepped is measured by the plane form or by plain kernels).
 static double sums_correction(const qf_lattice* lat, bool step) {
@@ -597,7 +601,10 @@ static FftPassArgs<R> fft_args(qf_lattice* lat, void* in, bool write, bool reduc
   p.data = reinterpret_cast<cpx<R>*>(lat->tmp());
   if constexpr (sizeof(R) == 4) {
     p.line = write && uses_line(lat) ? 1 : 0;
-    if (p.line || (uses_fft2(lat) && plane_supported(lat->d.n))) form_dtau(lat, p.tcoef, &p.dtau, &p.dtau_lo);
+    if (p.line || (uses_fft2(lat) && plane_supported(lat->d.n))) {
+      form_dtau(lat, p.tcoef, &p.dtau, &p.dtau_lo);
+      form_rest(lat, p.tcoef, &p.t0, &p.t0_lo);
+    }
   }
   return p;
 }
@@ -616,6 +623,7 @@ static ResArgs res_args(qf_lattice* lat, const double* scale, int nsteps) {
   r.am2 = p.am2;
   r.half_dtau = p.half_dtau;
   form_dtau(lat, p.tcoef, &r.dtau, &r.dtau_lo);
+  form_rest(lat, p.tcoef, &r.t0, &r.t0_lo);
   r.err = &lat->sc()->err[0];
   r.kinetic = p.kinetic;
   r.nsteps = nsteps;

@@ -84,10 +84,12 @@ struct FftPassArgs {
   cpx<R>* psi;            // psi_t in, psi_{t+1} out (same sites)
   const void* v;          // potential: cpx<R> (complex) or R (real)
   int v_real;
+  R t0;                   // resident, plane and line forms: rest mass left out of T(k) (rest_mass; else 0)
   const R* coef_u;        // complex FP64 and real V: 1 - coef_A per site (else null)
   R half_dtau;            // dtau / 2
   R dtau;
-  R dtau_lo;              // second part of dtau in the plane form (else unused)
+  R dtau_lo;              // second part of dtau in those forms (else unused)
+  R t0_lo;                // second part of t0
   const double* scale;    // output scale (device scalar)
   double* partials;       // per-block FP64 sums when reducing
   int write_psi;          // 0: measure only (no write)

@@ -115,10 +115,10 @@ __global__ void __launch_bounds__(LineG<N>::Z_THREADS) line_z_kernel(const __gri
   auto at = [&](int i) { return buf + 8 * i + c; };
   auto sync = [] { __syncthreads(); };
   line_fft<N, false>(v, g, tw_s, at, sync);
-  const float sxy = sym[kx] + sym[ky];
+  const float sxy = sym[kx] + sym[ky], am = sqrtf(a.am2);
 #pragma unroll
   for (int m = 0; m < E; ++m)
-    v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[g + G * m], a.tcoef, a.am2));
+    v[m] = cscale<float>(v[m], kin_mult_rest(a.kinetic, sxy, sym[g + G * m], a.tcoef, a.am2, am));
   line_fft<N, true>(v, g, tw_s, at, sync);
 #pragma unroll
   for (int m = 0; m < E; ++m) S[(long long)(g + G * m) * N * N] = v[m];
@@ -158,6 +158,10 @@ __global__ void __launch_bounds__(32 * LineG<N>::X_WARPS, LineG<N>::X_PER_SM)
   auto sync = [] { __syncwarp(); };
   line_fft<N, true>(v, g, tw_s, at, sync);
   // v = H_K psi (1/N^3 inside T)
+  if (N == 192 && a.kinetic == KIN_FFT_REL) {  // (the z pass of 512 is the four-pass kernel's, with all of T)
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = rest_mass(psi[m], v[m], a.t0, a.t0_lo);
+  }
   if constexpr (SUMS) {
     CheckSums<float> cs;
 #pragma unroll

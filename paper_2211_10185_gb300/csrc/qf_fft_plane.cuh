@@ -208,9 +208,10 @@ __global__ void __launch_bounds__(32 * PlaneG<N>::Z_WARPS) plane_z_kernel(const 
                               a.partials + (long long)(row0 + blockIdx.x) * kPartialStride);
     return;
   }
+  const float am = sqrtf(a.am2);
 #pragma unroll
   for (int m = 0; m < E; ++m)
-    v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[g + 4 * m], a.tcoef, a.am2));
+    v[m] = cscale<float>(v[m], kin_mult_rest(a.kinetic, sxy, sym[g + 4 * m], a.tcoef, a.am2, am));
   plane_line<N, true>(v, g, tw_s, at);
 #pragma unroll
   for (int m = 0; m < E; ++m) S[(long long)(g + 4 * m) * N * N] = v[m];
@@ -267,6 +268,10 @@ __global__ void __launch_bounds__(PlaneG<N>::P_THREADS) plane_p_kernel(const __g
   for (int m = 0; m < E; ++m) v[m] = *x_at(xg + 4 * m);
   plane_line<N, true>(v, xg, tw_s, x_at);
   // v = H_K psi (1/N^3 inside T)
+  if (a.kinetic == KIN_FFT_REL) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = rest_mass(psi[m], v[m], a.t0, a.t0_lo);
+  }
   if constexpr (SUMS) {
     CheckSums<float> cs;
 #pragma unroll

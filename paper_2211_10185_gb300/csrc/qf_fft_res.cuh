@@ -39,7 +39,7 @@ struct ResArgs {
   const double* scale;       // output scale of the first step
   const double* scale2;      // and of the others
   double* partials;          // kNumSums per block of the cluster when reducing
-  float tcoef, am2, half_dtau, dtau, dtau_lo;
+  float tcoef, am2, half_dtau, dtau, dtau_lo, t0, t0_lo;
   int* err;                  // set to 1 when a bounded wait ran out
   int kinetic, nsteps;
   unsigned spin;             // tries of a wait (kResSpin)
@@ -172,6 +172,7 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
   }
   bool ok = true;
   unsigned parity = 0;
+  const float am = sqrtf(a.am2);
   plane_twiddles<N>(tw_s, G::THREADS);
   for (int i = tid; i < N; i += G::THREADS) sym[i] = sym_g[i];
   const int s = tid / ST, warp = (tid % ST) >> 5, lane = tid & 31;
@@ -224,7 +225,7 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
     const float sxy = sym[col] + sym[rank * P + s];
 #pragma unroll
     for (int m = 0; m < E; ++m)
-      v[m] = cscale<float>(v[m], kin_mult_acc(a.kinetic, sxy, sym[cg + 4 * m], a.tcoef, a.am2));
+      v[m] = cscale<float>(v[m], kin_mult_rest(a.kinetic, sxy, sym[cg + 4 * m], a.tcoef, a.am2, am));
     plane_line<N, true>(v, cg, tw_s, z_at);
     __syncwarp();  // (as above)
     if (ok) {
@@ -247,6 +248,10 @@ __device__ __forceinline__ void res_body4(const ResArgs& a, const float* sym_g, 
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = *x_at(xg + 4 * m);
     plane_line<N, true>(v, xg, tw_s, x_at);
+    if (a.kinetic == KIN_FFT_REL) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) v[m] = rest_mass(psi[m], v[m], a.t0, a.t0_lo);
+    }
     if constexpr (SUMS) {
       CheckSums<float> sum;
 #pragma unroll
@@ -289,6 +294,7 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
   }
   bool ok = true;
   unsigned parity = 0;
+  const float am = sqrtf(a.am2);
   for (int i = tid; i < N; i += G::THREADS) sym[i] = sym_g[i];
   // the thread's line: row `l` of slab `s` as an x line, column `l` of slab s as a y or z line
   const int s = tid / N, l = tid % N;
@@ -341,7 +347,7 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
     }
     const float sxy = sym[l] + sym[rank * P + s];
 #pragma unroll
-    for (int z = 0; z < N; ++z) v[z] = cscale<float>(v[z], kin_mult_acc(a.kinetic, sxy, sym[z], a.tcoef, a.am2));
+    for (int z = 0; z < N; ++z) v[z] = cscale<float>(v[z], kin_mult_rest(a.kinetic, sxy, sym[z], a.tcoef, a.am2, am));
 #pragma unroll kUnroll
     for (int ph = 0; ph < 3; ++ph) {  // z, y, x inverse
       rc_dft<N, true, 1>(v);
@@ -365,6 +371,10 @@ __device__ __forceinline__ void res_body(const ResArgs& a, const float* sym_g, f
       }
     }
     // v = H_K psi at the sites of psi; update
+    if (a.kinetic == KIN_FFT_REL) {
+#pragma unroll
+      for (int x = 0; x < N; ++x) v[x] = rest_mass(psi[x], v[x], a.t0, a.t0_lo);
+    }
     if constexpr (SUMS) {
       CheckSums<float> sum;
 #pragma unroll

@@ -145,6 +145,7 @@ extern "C" qf_status qf_fft_step_static(int n, double a, int kinetic, double mas
     r.a.am2 = am2;
     r.a.half_dtau = (float)(0.5 * dtau);
     kinetic_dtau(n, 0, dtau, exact, tcoef, &r.a.dtau, &r.a.dtau_lo);
+    kinetic_rest(n, 0, mass, exact, tcoef, &r.a.t0, &r.a.t0_lo);
     r.a.kinetic = kinetic;
     r.a.nsteps = 1;
     r.a.spin = kResSpin;

@@ -56,3 +56,9 @@ def _check(n, kind, seed):
                                          (48, O.FFT_SYMANZIK, 4), (64, O.FFT_NAIVE, 2)])
 def test_narrow_fields_of_heavy_particles(n, kind, seed):
     _check(n, kind, seed)
+
+
+@pytest.mark.parametrize("n,seed", [(32, 18), (32, 1), (48, 4), (64, 1)])
+def test_heavy_relativistic_particles(n, seed):
+    """Eq. HK3 with T(k) close to the mass for all k that matter."""
+    _check(n, O.FFT_REL, seed)
