@@ -215,9 +215,9 @@ static bool uses_res(const qf_lattice* lat) {
 
 // Sizes whose form is the default.  N = 96 takes the four-pass form unless asked for: the plane
 // form's field and energy (a step in 17.9 us against 25.1) differ from the four-pass form's by the
-// roundings of both, 1e-7 of <T> at the start field and up to 1e-6 after 64 steps (the plane
-// form 1e-7 from 64-bit arithmetic, the four-pass form 8e-7), which is 1e-4 of E where <T> and <V>
-// nearly cancel; and at this size it holds 96 lines of two fields in registers and spills.
+// roundings of both, nearly all the latter's, 1e-7 of <T> at the start field and up to 1e-6 after
+// 64 steps, which is 1e-4 of E where <T> and <V> nearly cancel; and at this size it holds 96 lines
+// of two fields in registers and spills.
 static bool default_form(int n) { return n != 96; }
 
 static void drop_graphs(qf_lattice* lat) {

@@ -21,8 +21,8 @@
 //
 // What bounds it: the latency of a block's four transforms with 6-12 warps per SM, on N of the 152
 // SMs in P (the four-pass form: that of four launches, 11.6-25 us a step).  One step with
-// Eq. HK2 (of 64 with a check), before and now: N = 48: 12.8 / 5.8 us, 64: 11.6-13 / 8.7, 96: 25.1 /
-// 17.9 (not the default there).  N = 128 took 40 us so (32 elements a thread, one block of 16
+// Eq. HK2 (of 64 with a check), before and now: N = 48: 12.8 / 5.8 us, 64: 11.6-13 / 8.7 (Eq. HK3
+// 9.5), 96: 25.1 / 17.9 (not the default there).  N = 128 took 40 us so (32 elements a thread, one block of 16
 // warps per SM, spills) against 25.7 in the split form.
 #pragma once
 #include "qf_fft_reg.cuh"
